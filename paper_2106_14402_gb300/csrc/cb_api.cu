@@ -612,7 +612,7 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   mark(ctx, opt, 4);
   cb::launch_numeric(sr, dA, dB, perm_num, num_beg, num_cnt, flops, nnz, heavy_rows, wins,
                      n_units, span_counts, spans, hbits, b_sorted, C->row_ptr, C->col, C->val,
-                     counters + cb::kError, ctx->stream, ctx->sms, &launches, num_hash_max, racc,
+                     counters, ctx->stream, ctx->sms, &launches, num_hash_max, racc,
                      cb::CfBounds{ctx->tune.cf_esc, ctx->tune.cf_pre});
   CB_LAUNCHED();
   mark(ctx, opt, 5);

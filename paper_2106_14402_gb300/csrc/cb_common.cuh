@@ -416,6 +416,14 @@ __device__ __forceinline__ uint32_t hash_slot(int32_t c, int shift) {
   return ((uint32_t)c * 2654435769u) >> shift;
 }
 
+// Units of a persistent kernel, taken one after the other from a counter that
+// starts at zero: thread 0 puts the CTA's next unit into the shared *slot.
+// A barrier stands between the others' last read of the slot and this call,
+// another between the call and their next read.
+__device__ __forceinline__ void take_unit(int64_t* queue, long long* slot) {
+  if (threadIdx.x == 0) *slot = (long long)atomicAdd((unsigned long long*)queue, 1ull);
+}
+
 // Find the slot of key c in an open-addressing (linear probing) table of
 // mask+1 slots, inserting it if absent.  Returns the slot, or -1 if the
 // table is full (never happens for tables sized >= 2x the row bound).

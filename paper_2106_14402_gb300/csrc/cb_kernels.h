@@ -63,6 +63,9 @@ enum Counter {
   kUnsorted = 24,       // > 0 when some row of B is not non-decreasing
   kMaxFlops = 25,       // largest flops_i (k_classify_sym)
   kMaxArow = 26,        // longest row of A (k_classify_sym)
+  kCurHeavy = 27,       // scatter cursor of the heavy rows placed from the segment's end
+  kSymQueue = 28,       // next unit of the heavy rows' symbolic pass
+  kNumQueue = 29,       // next rank window of the numeric phase
   kCounters = 32
 };
 
@@ -150,7 +153,7 @@ void launch_numeric(int sr, const DevCSR& A, const DevCSR& B, const int32_t* per
                     const int64_t* nnz, const int32_t* heavy_rows, const Window* wins,
                     int64_t n_wins, const int32_t* span_counts, int64_t spans,
                     const unsigned* hbits, int b_sorted, const int64_t* Crp, int32_t* Ccol,
-                    void* Cval, int64_t* err, cudaStream_t s, int sms, int* launches,
+                    void* Cval, int64_t* counters, cudaStream_t s, int sms, int* launches,
                     int64_t num_hash_max = 512, void* racc = nullptr, CfBounds cf = {});
 
 // Batched products (cb_batched.cu): stack parts into one CSR.
@@ -231,7 +234,7 @@ void launch_symbolic_dev(const DevCSR& A, const DevCSR& B, const int32_t* perm, 
                          const int64_t* flops, int64_t* nnz, int32_t* span_counts, int2* span_wins,
                          int wcut, Window* wins, int64_t win_cap, cudaStream_t s, int sms);
 void launch_numeric_dev(int sr, const DevCSR& A, const DevCSR& B, const int32_t* perm,
-                        const int64_t* counters, const int64_t* flops, const int64_t* nnz,
+                        int64_t* counters, const int64_t* flops, const int64_t* nnz,
                         const int64_t* Crp, int32_t* Ccol, void* Cval, int64_t* err, cudaStream_t s,
                         int sms, const int32_t* perm_sym, const Window* wins,
                         const int32_t* span_counts, int64_t spans, void* racc, int64_t num_hash_max,

@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(CTA) k_num_hash(DevCSR A, DevCSR B, const int3
 // window's column bitmap (stored by the symbolic phase, or rebuilt from the
 // row's products), prefix-count its words, then accumulate every product
 // into the dense accumulator at its column's rank and write the window's
-// slice of the row in column order.
+// slice of the row in column order.  Windows are taken from a queue.
 constexpr bool kRankInPlace = true;
 
 // Launch shape of the rank windows per semiring: 512-thread CTAs, three per
@@ -306,7 +306,7 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
                                                       const int64_t* flops, const int64_t* nnz,
                                                       const int64_t* Crp, int32_t* Ccol,
                                                       typename Sem<SR>::TC* Cval, int64_t* err,
-                                                      int64_t num_hash_max,
+                                                      int64_t* queue, int64_t num_hash_max,
                                                       typename Sem<SR>::A* racc,
                                                       const int64_t* dcounters = nullptr) {
   typedef Sem<SR> S;
@@ -351,14 +351,22 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
   const PieceSmem sm{reinterpret_cast<int*>(bal + 2 * CTA), bal, bal + CTA,
                      reinterpret_cast<int*>(bal + 2 * CTA) + CTA, scan64};
   __shared__ long long s_base;
+  __shared__ long long next;
   const int tid = threadIdx.x, lane = tid & 31;
   const TA* Aval = reinterpret_cast<const TA*>(A.val);
   const TB* Bval = reinterpret_cast<const TB*>(B.val);
 
-  for (int64_t u = blockIdx.x; u < n_wins; u += gridDim.x) {
+  take_unit(queue, &next);
+  __syncthreads();
+  for (int64_t u = next; u < n_wins; u = next) {
     const Window wd = wins[u];
     const int i = heavy_rows[wd.h];
-    if (nnz[i] <= num_hash_max || wd.count <= 0) continue;  // hash tiers own these rows
+    if (nnz[i] <= num_hash_max || wd.count <= 0) {  // hash tiers own these rows
+      __syncthreads();  // every thread has read this unit
+      take_unit(queue, &next);
+      __syncthreads();
+      continue;
+    }
     const int cnt = wd.count < WCAP ? wd.count : WCAP;
     const int64_t span_lo = B.col_lo + (int64_t)wd.span * kSpanCols;
     const int64_t lo = span_lo + 32 * (int64_t)wd.w_lo;
@@ -467,6 +475,7 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
       const int64_t o = out + j;
       if (guard(o < row_end, 39, o)) st_out(Ccol + o, (int32_t)(lo + c));
     });
+    take_unit(queue, &next);
     __syncthreads();
   }
 }
@@ -486,11 +495,12 @@ void numeric_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, const int
                 const int64_t* seg_count, const int64_t* flops, const int64_t* nnz,
                 const int32_t* heavy_rows, const Window* wins, int64_t n_wins,
                 const int32_t* span_counts, int64_t spans, const unsigned* hbits, int b_sorted,
-                const int64_t* Crp, int32_t* Ccol, void* Cval_, int64_t* err, cudaStream_t s,
+                const int64_t* Crp, int32_t* Ccol, void* Cval_, int64_t* counters, cudaStream_t s,
                 int sms, int* launches, int64_t num_hash_max, void* racc, CfBounds cf) {
   typedef typename Sem<SR>::A Acc;
   typedef typename Sem<SR>::TC TC;
   TC* Cval = reinterpret_cast<TC*>(Cval_);
+  int64_t* err = counters + kError;
   constexpr size_t slot = sizeof(Acc) + sizeof(int);
   if (seg_count[kNumWarp]) {
     constexpr int CTA = 256, TEAM = 32, TBL = 2 * kNumWarpMax;
@@ -526,7 +536,7 @@ void numeric_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, const int
     set_smem(k_num_rank<SR, CTA>, smem);
     k_num_rank<SR, CTA><<<capped(n_wins, (int64_t)sms * PER_SM), CTA, smem, s>>>(
         A, B, heavy_rows, wins, n_wins, span_counts, spans, hbits, b_sorted, flops, nnz, Crp, Ccol,
-        Cval, err, num_hash_max, static_cast<Acc*>(racc));
+        Cval, err, counters + kNumQueue, num_hash_max, static_cast<Acc*>(racc));
     ++*launches;
   }
 }
@@ -534,7 +544,7 @@ void numeric_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, const int
 // Hash tiers only, tier sizes read on the device (counters[kCntNum..]): the
 // grids are sized for the worst case and the kernels stride over their tier.
 template <int SR>
-void numeric_dev_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, const int64_t* counters,
+void numeric_dev_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, int64_t* counters,
                     const int64_t* flops, const int64_t* nnz, const int64_t* Crp, int32_t* Ccol,
                     void* Cval_, int64_t* err, cudaStream_t s, int sms, int64_t m,
                     const int32_t* perm_sym, const Window* wins, const int32_t* span_counts,
@@ -567,7 +577,7 @@ void numeric_dev_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, const
     constexpr size_t smem = RankShape<SR>::kSmem;
     k_num_rank<SR, CTA><<<sms * PER_SM, CTA, smem, s>>>(
         A, B, perm_sym, wins, 0, span_counts, spans, nullptr, 0, flops, nnz, Crp, Ccol, Cval, err,
-        num_hash_max, static_cast<Acc*>(racc), counters);
+        counters + kNumQueue, num_hash_max, static_cast<Acc*>(racc), counters);
   }
 }
 
@@ -656,11 +666,11 @@ void launch_numeric(int sr, const DevCSR& A, const DevCSR& B, const int32_t* per
                     const int64_t* nnz, const int32_t* heavy_rows, const Window* wins,
                     int64_t n_wins, const int32_t* span_counts, int64_t spans,
                     const unsigned* hbits, int b_sorted, const int64_t* Crp, int32_t* Ccol,
-                    void* Cval, int64_t* err, cudaStream_t s, int sms, int* launches,
+                    void* Cval, int64_t* counters, cudaStream_t s, int sms, int* launches,
                     int64_t num_hash_max, void* racc, CfBounds cf) {
 #define CB_NUM(SRV)                                                                        \
   numeric_sr<SRV>(A, B, perm, seg_begin, seg_count, flops, nnz, heavy_rows, wins, n_wins,   \
-                  span_counts, spans, hbits, b_sorted, Crp, Ccol, Cval, err, s, sms, launches, \
+                  span_counts, spans, hbits, b_sorted, Crp, Ccol, Cval, counters, s, sms, launches, \
                   num_hash_max, racc, cf)
   switch (sr) {
 #define CB_CASE(SRV) case SRV: CB_NUM(SRV); break;
@@ -698,7 +708,7 @@ void prepare_dev_launchers(int sr) {
 }
 
 void launch_numeric_dev(int sr, const DevCSR& A, const DevCSR& B, const int32_t* perm,
-                        const int64_t* counters, const int64_t* flops, const int64_t* nnz,
+                        int64_t* counters, const int64_t* flops, const int64_t* nnz,
                         const int64_t* Crp, int32_t* Ccol, void* Cval, int64_t* err, cudaStream_t s,
                         int sms, const int32_t* perm_sym, const Window* wins,
                         const int32_t* span_counts, int64_t spans, void* racc, int64_t num_hash_max,

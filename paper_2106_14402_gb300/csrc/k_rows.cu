@@ -84,6 +84,7 @@ struct TierBySize {
   int64_t cap, t1, t2, t3;
   const uint8_t* skip;         // rows with skip[i] != 0 are left out (tier 0)
   const int32_t* rcap = nullptr;  // per-row cap (replaces cap when set)
+  int64_t* counters = nullptr;    // symbolic tiers: tier 4 in two classes (k_tier_scatter)
   __device__ __forceinline__ int operator()(int64_t i) const {
     if (skip && skip[i]) return 0;
     const int64_t u = min(v[i], rcap ? (int64_t)rcap[i] : cap);
@@ -107,12 +108,19 @@ __global__ void __launch_bounds__(256) k_tier_count(int64_t m, TierBySize tier, 
 // order; tier 0 rows are empty or skipped and get no slot).  zero_nnz
 // (optional): rows of tier 0 and 4 get nnz = 0 (tier 4 rows are summed slice
 // by slice later), except skipped rows, which get preset[i].
+// Symbolic tiers (tier.counters set) order tier 4, whose rows the persistent
+// kernels take one after the other: rows with at least 1/2^kBigShift of all
+// products fill the segment from its front, the others from its back, so the
+// last units handed out are small.  On R-MAT s18 (304 CTAs; hub rows of up to
+// 8M of 9.5G products anywhere in the order, units assigned in a fixed
+// stride) the busy time of all CTAs was 77-84% of the kernels' time.
+constexpr int kBigShift = 14;
 __global__ void __launch_bounds__(256) k_tier_scatter(int64_t m, TierBySize tier, int32_t* perm,
                                                       const int64_t* cnt, int64_t* cur,
                                                       int64_t* zero_nnz, const int64_t* preset) {
-  __shared__ int local[5];
-  __shared__ long long base[5];
-  if (threadIdx.x < 5) local[threadIdx.x] = 0;
+  __shared__ int local[6];  // tiers; 5 = the rows of tier 4 placed from its end
+  __shared__ long long base[6];
+  if (threadIdx.x < 6) local[threadIdx.x] = 0;
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int t = -1, slot = 0;
@@ -122,6 +130,7 @@ __global__ void __launch_bounds__(256) k_tier_scatter(int64_t m, TierBySize tier
       if (tier.skip && tier.skip[i]) zero_nnz[i] = preset ? preset[i] : 0;
       else if (t == 0 || t == 4) zero_nnz[i] = 0;
     }
+    if (t == 4 && tier.counters && tier.v[i] < (tier.counters[kTotalFlops] >> kBigShift)) t = 5;
     if (t > 0) slot = atomicAdd(&local[t], 1);
   }
   __syncthreads();
@@ -132,7 +141,12 @@ __global__ void __launch_bounds__(256) k_tier_scatter(int64_t m, TierBySize tier
         seg + (long long)atomicAdd((unsigned long long*)&cur[threadIdx.x], (unsigned long long)local[threadIdx.x]);
   }
   __syncthreads();
-  if (t > 0) perm[base[t] + slot] = (int32_t)i;
+  if (threadIdx.x == 5 && local[5])
+    base[5] = cnt[1] + cnt[2] + cnt[3] + cnt[4] - 1 -
+              (long long)atomicAdd((unsigned long long*)&tier.counters[kCurHeavy], (unsigned long long)local[5]);
+  __syncthreads();
+  if (t == 5) perm[base[5] - slot] = (int32_t)i;
+  else if (t > 0) perm[base[t] + slot] = (int32_t)i;
 }
 
 // K4: three-pass exclusive scan (tile reduce, scan of tile sums, apply).
@@ -268,7 +282,7 @@ void launch_scatter_sym(int64_t m, int64_t ncols, const int64_t* flops, int32_t*
                         int64_t* nnz, int64_t* counters, cudaStream_t s, int,
                         const uint8_t* skip, const int64_t* preset, int64_t sym_hash_max,
                         const int32_t* rcols) {
-  TierBySize t{flops, ncols, kSymWarpMax, kSymSmallMax, sym_hash_max, skip, rcols};
+  TierBySize t{flops, ncols, kSymWarpMax, kSymSmallMax, sym_hash_max, skip, rcols, counters};
   k_tier_scatter<<<grid_for(m, 256, 1 << 30), 256, 0, s>>>(m, t, perm, counters + kCntSym,
                                                             counters + kCurSym, nnz, preset);
 }

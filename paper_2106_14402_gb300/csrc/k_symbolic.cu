@@ -75,7 +75,7 @@ __global__ void __launch_bounds__(CTA) k_sym_hash(DevCSR A, DevCSR B, const int3
 // Heavy rows (u > 512): one CTA per (heavy row h, span) unit.  The bitmap
 // covers the span's columns [lo, hi); after counting, the span is cut into
 // rank windows of at most wcut + 31 entries (see cb_common.cuh), appended to
-// `wins` (when non-null) for the numeric phase.
+// `wins` (when non-null) for the numeric phase.  Units are taken from a queue.
 __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, const int32_t* heavy_rows,
                                                      int64_t n_heavy, int64_t spans,
                                                      const int64_t* flops, int wcut, int64_t* nnz,
@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
   __shared__ int wstart[kMaxWindowsPerSpan];
   __shared__ int wrank[kMaxWindowsPerSpan];
   __shared__ long long wbase;
+  __shared__ long long next;
   constexpr int WPT = kSpanWords / 1024;  // bitmap words per thread in the scan
   const int tid = threadIdx.x;
   if (b_sorted < 0) {  // sizes on the device: heavy segment of perm, count, B's sortedness
@@ -104,8 +105,9 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
   // the bitmap starts clear; each unit clears the words it set once it has
   // read them, so no unit starts with a clearing pass of its own
   for (int w = tid; w < bm_words; w += 1024) sym_bm[w] = 0u;
+  take_unit(counters + kSymQueue, &next);
   __syncthreads();
-  for (int64_t u = blockIdx.x; u < units; u += gridDim.x) {
+  for (int64_t u = next; u < units; u = next) {
     const int64_t h = spans == 1 ? u : u / spans, sp = u - h * spans;
     const int i = heavy_rows[h];
     const int64_t lo = B.col_lo + sp * (int64_t)kSpanCols;
@@ -115,6 +117,9 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
         span_counts[h * spans + sp] = 0;
         if (span_wins) span_wins[h * spans + sp] = make_int2(0, 0);
       }
+      __syncthreads();  // every thread has read this unit
+      take_unit(counters + kSymQueue, &next);
+      __syncthreads();
       continue;
     }
     const int nwords = (int)((hi - lo + 31) / 32);
@@ -202,6 +207,7 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
       if (total) atomicAdd((unsigned long long*)&nnz[i], (unsigned long long)total);
     }
     for (int w = tid; w < nwords; w += 1024) sym_bm[w] = 0u;  // every read of them is done
+    take_unit(counters + kSymQueue, &next);
     __syncthreads();
   }
 }
