@@ -530,9 +530,8 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
 
   const int64_t n_heavy = sym_cnt[cb::kSymHeavy];
   const int64_t spans = (ncols + cb::kSpanCols - 1) / cb::kSpanCols;
-  const int wcut = cb::num_window_cut(sr);
-  // every (row, span) yields at most count/wcut + 1 windows; counts sum to <= flops
-  const int64_t win_cap = n_heavy * spans + ctx->stats.flops / wcut + 1;
+  const cb::WinCut wcut = cb::num_window_cut(sr);
+  const int64_t win_cap = wcut.most(n_heavy * spans, cb::kSpanWords, ctx->stats.flops);
 
   // Heavy-row bitmaps are kept for the numeric phase when they fit a quarter
   // of free device memory (capped at 32 GiB); otherwise the numeric phase
@@ -542,10 +541,14 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   CB_CUDA(cudaMemGetInfo(&free_b, &total_b));
   const bool keep_bits = n_heavy > 0 && bits_bytes <= free_b / 4 && bits_bytes <= (32ull << 30);
   const size_t racc_bytes = n_heavy > 0 ? cb::rank_scratch_bytes(sr, ctx->sms) : 0;
+  // rank windows that cover part of a row slice B's rows by a split table
+  size_t tab_bytes = 0;
+  cb::SplitTable tab;
+  if (n_heavy > 0 && b_sorted) tab = cb::split_table_shape(dB.nrows, ncols, &tab_bytes);
   size_t need2 = align_up(4 * (size_t)(n_heavy * spans) + 4) +
                  align_up(8 * (size_t)(n_heavy * spans) + 8) +
                  align_up(sizeof(cb::Window) * (size_t)win_cap) + (keep_bits ? align_up(bits_bytes) : 0) +
-                 align_up(racc_bytes);
+                 align_up(racc_bytes) + align_up(tab_bytes);
   ensure(ctx, &ctx->ws2, &ctx->ws2_cap, need2);
   Carver cv2{static_cast<char*>(ctx->ws2)};
   int32_t* span_counts = cv2.take<int32_t>(n_heavy * spans + 1);
@@ -553,6 +556,7 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   cb::Window* wins = cv2.take<cb::Window>(win_cap);
   unsigned* hbits = keep_bits ? cv2.take<unsigned>((size_t)(n_heavy * spans) * cb::kSpanWords) : nullptr;
   void* racc = racc_bytes ? cv2.take<char>(racc_bytes) : nullptr;
+  int32_t* tab_pos = tab_bytes ? cv2.take<int32_t>(tab_bytes / 4) : nullptr;
   const int32_t* heavy_rows = perm_sym + sym_beg[cb::kSymHeavy];
 
   int launches = 0;
@@ -610,10 +614,17 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
 
   launches = 0;
   mark(ctx, opt, 4);
+  // a pass over B's rows for the table pays once more than a few rows are cut
+  // into several windows (a row's only window takes B's rows whole)
+  if (tab_pos && n_units > n_heavy + n_heavy / 8) {
+    tab.pos = tab_pos;
+    cb::launch_split_table(dB, tab, ctx->stream, ctx->sms);
+    ++launches;
+  }
   cb::launch_numeric(sr, dA, dB, perm_num, num_beg, num_cnt, flops, nnz, heavy_rows, wins,
                      n_units, span_counts, spans, hbits, b_sorted, C->row_ptr, C->col, C->val,
                      counters, ctx->stream, ctx->sms, &launches, num_hash_max, racc,
-                     cb::CfBounds{ctx->tune.cf_esc, ctx->tune.cf_pre});
+                     cb::CfBounds{ctx->tune.cf_esc, ctx->tune.cf_pre}, tab);
   CB_LAUNCHED();
   mark(ctx, opt, 5);
   ctx->stats.kernels += launches;
@@ -1083,7 +1094,7 @@ bool batched_group_graph(cb_ctx* ctx, int sr, const cb_csr& sA, const DevCSR& dB
   const int64_t sym_max = ctx->tune.sym_hash_max;
   const int64_t num_max = std::min<int64_t>(ctx->tune.num_hash_max, cb::num_large_max(sr));
   const int64_t spans = (kmax + cb::kSpanCols - 1) / cb::kSpanCols;
-  const int wcut = cb::num_window_cut(sr);
+  const cb::WinCut wcut = cb::num_window_cut(sr);
   // waves by the flop bound
   std::vector<int> cut{0};
   int64_t rows = 0, nz = 0;
@@ -1109,8 +1120,7 @@ bool batched_group_graph(cb_ctx* ctx, int sr, const cb_csr& sA, const DevCSR& dB
     int64_t f = 0;
     for (int i = cut[w]; i < cut[w + 1]; ++i) f += sizes[(size_t)i];
     max_cap = std::max(max_cap, f);
-    // every (row, span) yields at most count / wcut + 1 windows; counts sum to <= flops
-    max_wins = std::max(max_wins, r * spans + f / wcut + 1);
+    max_wins = std::max(max_wins, wcut.most(r * spans, cb::kSpanWords, f));
   }
   // everything the graph touches is allocated before the capture
   DevBuf orp(ctx), ocol(ctx), oval(ctx), wsb(ctx), errw(ctx), dscr(ctx);

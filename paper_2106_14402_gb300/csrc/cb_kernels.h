@@ -32,6 +32,26 @@ struct CfBounds {
 
 struct Window;
 
+// How the symbolic phase cuts a span's bitmap into rank windows: word w opens
+// a new window where per_word * w + per_entry * (entries before w) crosses a
+// multiple of `cut`, so a window weighs at most cut + per_word + 32 * per_entry.
+struct WinCut {
+  int cut = 1, per_word = 0, per_entry = 1;
+  // windows of `units` (row, span) pairs of span_words words holding at most `entries`
+  int64_t most(int64_t units, int64_t span_words, int64_t entries) const {
+    return units * (1 + (per_word * span_words + cut - 1) / cut) + per_entry * entries / cut + 1;
+  }
+};
+
+// Where each row of a sorted B crosses the multiples of 2^shift columns of its
+// view: entry g of row k (stride entries a row) counts the row's entries
+// before column col_lo + (g << shift); the last entry is the row's length.
+// pos == nullptr: no table.
+struct SplitTable {
+  const int32_t* pos = nullptr;
+  int stride = 0, shift = 0;
+};
+
 // A CSR operand as the kernels see it.  For B it may be a column window:
 // only columns in [col_lo, col_lo + ncols) belong to the view.  Row k spans
 // [rp[k], rpe[k]) (rpe == nullptr: rp[k + 1]).  With filter == 0 every entry
@@ -106,6 +126,12 @@ void launch_gather(const int64_t* prefix, const int64_t* idx, int64_t n, int64_t
 void launch_slabs(const DevCSR& B, const int64_t* bnd, int nb1, int64_t* pos, cudaStream_t s,
                   int sms);
 
+// Shape of a split table for a view of n rows and ncols columns (pos unset)
+// and its bytes; stride 0 where a table would not pay.
+SplitTable split_table_shape(int64_t n, int64_t ncols, size_t* bytes);
+// Fills the table t (t.pos is device memory of that size); B's rows must be sorted.
+void launch_split_table(const DevCSR& B, const SplitTable& t, cudaStream_t s, int sms);
+
 // Numeric binning by exact row size.
 void launch_classify_num(int sr, int64_t m, const int64_t* nnz, int32_t* perm,
                          int64_t* counters, cudaStream_t s, int sms,
@@ -132,13 +158,13 @@ void launch_compact_rows(int vsz, int64_t m, const uint8_t* learned, const int64
 // K3: symbolic phase, all tiers.  perm holds the tier segments in order;
 // seg_begin[t] / seg_count[t] are host copies of the tier layout.  Heavy
 // rows (tier 4) write span_counts[h * spans + span] and, when wins is
-// non-null, append their rank windows (cut every `wcut` entries) to wins
+// non-null, append their rank windows (cut by `wcut`) to wins
 // (capacity win_cap; counters[kUnits] counts them).
 // (span_wins[h * spans + span] = {first window, window count}; hbits, when
 // non-null, receives each heavy row's bitmap: kSpanWords words per (row, span).)
 void launch_symbolic(const DevCSR& A, const DevCSR& B, const int32_t* perm,
                      const int64_t* seg_begin, const int64_t* seg_count, const int64_t* flops,
-                     int64_t* nnz, int32_t* span_counts, int2* span_wins, int wcut,
+                     int64_t* nnz, int32_t* span_counts, int2* span_wins, WinCut wcut,
                      Window* wins, int64_t win_cap, unsigned* hbits, int b_sorted,
                      int64_t* counters, cudaStream_t s, int sms, int* launches);
 // Sets counters[kUnsorted] > 0 if some row of B decreases in column.
@@ -146,7 +172,7 @@ void launch_check_sorted(const DevCSR& B, int64_t* counters, cudaStream_t s, int
 
 // K5-K7: numeric phase over the numeric tier segments + rank windows,
 // writing sorted rows of C at Crp.
-int num_window_cut(int sr);
+WinCut num_window_cut(int sr);
 int num_large_max(int sr);
 void launch_numeric(int sr, const DevCSR& A, const DevCSR& B, const int32_t* perm,
                     const int64_t* seg_begin, const int64_t* seg_count, const int64_t* flops,
@@ -154,7 +180,8 @@ void launch_numeric(int sr, const DevCSR& A, const DevCSR& B, const int32_t* per
                     int64_t n_wins, const int32_t* span_counts, int64_t spans,
                     const unsigned* hbits, int b_sorted, const int64_t* Crp, int32_t* Ccol,
                     void* Cval, int64_t* counters, cudaStream_t s, int sms, int* launches,
-                    int64_t num_hash_max = 512, void* racc = nullptr, CfBounds cf = {});
+                    int64_t num_hash_max = 512, void* racc = nullptr, CfBounds cf = {},
+                    const SplitTable& tab = {});
 
 // Batched products (cb_batched.cu): stack parts into one CSR.
 size_t stack_part_size();
@@ -232,7 +259,7 @@ void prepare_symbolic_dev();
 void prepare_dev_launchers(int sr);  // sets the shared-memory attributes of both (not capturable)
 void launch_symbolic_dev(const DevCSR& A, const DevCSR& B, const int32_t* perm, int64_t* counters,
                          const int64_t* flops, int64_t* nnz, int32_t* span_counts, int2* span_wins,
-                         int wcut, Window* wins, int64_t win_cap, cudaStream_t s, int sms);
+                         WinCut wcut, Window* wins, int64_t win_cap, cudaStream_t s, int sms);
 void launch_numeric_dev(int sr, const DevCSR& A, const DevCSR& B, const int32_t* perm,
                         int64_t* counters, const int64_t* flops, const int64_t* nnz,
                         const int64_t* Crp, int32_t* Ccol, void* Cval, int64_t* err, cudaStream_t s,

@@ -257,20 +257,30 @@ __global__ void __launch_bounds__(CTA) k_num_hash(DevCSR A, DevCSR B, const int3
 // slice of the row in column order.  Windows are taken from a queue.
 constexpr bool kRankInPlace = true;
 
-// Launch shape of the rank windows per semiring: 512-thread CTAs, three per
-// SM, when the accumulators take little or no shared memory (8-byte ones
-// reduce in L2; (or,and) keeps one bit per slot), else one 1024-thread CTA
-// per SM holding kWcap 4-byte shared accumulators.
+// Launch shape of the rank windows: three 512-thread CTAs per SM, so that one
+// window's setup, searches and read-out overlap the others' products.
+//   * 8-byte accumulators reduce in L2 (a window holds at most kWcap entries);
+//     (or,and) keeps one bit per slot; both hold a whole span's words.
+//   * 4-byte ones share a pool of kWinPool bytes with the window's words
+//     (6 bytes a word, 4 an entry): sparse rows get many words and few
+//     entries, dense rows the reverse.  (With 32768 accumulators beside a
+//     span's words, one 1024-thread CTA per SM, 64% of a window's time was
+//     setup, search and read-out with nothing to overlap it.  R-MAT s14
+//     select2nd 0.76 -> 0.55 ms; s18 u32, twice as many windows, 37.0 -> 34.0
+//     ms together with the split table, 36.8 without it.)
 template <int SR>
 struct RankShape {
   static constexpr bool kBits = SR == 4;
-  static constexpr int kCta = (NumLimits<SR>::kL2Acc || kBits) ? 512 : 1024;
-  static constexpr size_t kAccBytes =
-      NumLimits<SR>::kL2Acc ? 0
-      : kBits ? (size_t)NumLimits<SR>::kWcap / 8
-              : (size_t)NumLimits<SR>::kWcap * sizeof(typename Sem<SR>::A);
-  static constexpr size_t kSmem = kAccBytes + kSpanWords * (sizeof(unsigned) + sizeof(unsigned short)) +
-                                  (size_t)kCta * PieceSmem::kBytesPerThread;
+  static constexpr bool kPool = !NumLimits<SR>::kL2Acc && !kBits;
+  static constexpr int kCta = 512, kPerSm = 3;
+  static constexpr size_t kAccBytes = kBits ? (size_t)NumLimits<SR>::kWcap / 8 : 0;
+  static constexpr size_t kWordBytes =
+      kPool ? (size_t)kWinPool : kSpanWords * (sizeof(unsigned) + sizeof(unsigned short));
+  static constexpr size_t kSmem = kAccBytes + kWordBytes + (size_t)kCta * PieceSmem::kBytesPerThread;
+  // entries: kWcap less the words the last one may overshoot by; pool: less a
+  // word's weight and the rounding of the words to 8
+  static constexpr WinCut kCut =
+      kPool ? WinCut{kWinPool - (6 + 32 * 4) - 7 * 6, 6, 4} : WinCut{NumLimits<SR>::kWcap - 32, 0, 1};
 };
 
 // L2 residency of the windows that accumulate in C (fp64 and int64): the
@@ -299,7 +309,8 @@ __device__ __forceinline__ void demote_line(const void* a) {
 }
 
 template <int SR, int CTA>
-__global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, DevCSR B, const int32_t* heavy_rows,
+__global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR A, DevCSR B, SplitTable tab,
+                                                      const int32_t* heavy_rows,
                                                       const Window* wins, int64_t n_wins,
                                                       const int32_t* span_counts, int64_t spans,
                                                       const unsigned* hbits, int b_sorted,
@@ -334,8 +345,8 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
   constexpr int WPT = kSpanWords / CTA;
   static_assert(WCAP <= 65535, "a window's entry counts are kept in 16 bits");
   extern __shared__ __align__(16) unsigned char rank_smem[];
-  // shared layout: [accumulators (shared-memory windows only)] [bx] [by] [iterator scratch]
-  Acc* acc = reinterpret_cast<Acc*>(rank_smem);
+  // shared layout: [(or,and) bits] [bx] [by] [4-byte accumulators] [iterator scratch];
+  // in a pool, by and the accumulators start behind the window's own words
   // word w of the window: bx[w] = its column bits, by[w] = entries of the
   // window before it (< 2^16: a window holds at most kWcap entries).  Two
   // arrays, not one of pairs: a product's lookup of both words then meets
@@ -344,8 +355,10 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
   constexpr bool kBits = RankShape<SR>::kBits;  // (or,and): one accumulator bit per slot
   unsigned* accbits = reinterpret_cast<unsigned*>(rank_smem);
   unsigned* bx = reinterpret_cast<unsigned*>(rank_smem + RankShape<SR>::kAccBytes);
+  constexpr bool kPool = RankShape<SR>::kPool;
   unsigned short* by = reinterpret_cast<unsigned short*>(bx + kSpanWords);
-  long long* bal = reinterpret_cast<long long*>(by + kSpanWords);
+  Acc* acc = nullptr;
+  long long* bal = reinterpret_cast<long long*>(rank_smem + RankShape<SR>::kAccBytes + RankShape<SR>::kWordBytes);
   __shared__ int scratch[33];
   __shared__ long long scan64[33];
   const PieceSmem sm{reinterpret_cast<int*>(bal + 2 * CTA), bal, bal + CTA,
@@ -367,13 +380,19 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
       __syncthreads();
       continue;
     }
-    const int cnt = wd.count < WCAP ? wd.count : WCAP;
+    int cnt = wd.count < WCAP ? wd.count : WCAP;
     const int64_t span_lo = B.col_lo + (int64_t)wd.span * kSpanCols;
     const int64_t lo = span_lo + 32 * (int64_t)wd.w_lo;
     const int64_t rw = row_width(A, B, i);
     const int64_t hi = min(span_lo + 32 * (int64_t)wd.w_hi, B.col_lo + rw);
     const bool whole = lo == B.col_lo && hi == B.col_lo + rw && !B.filter;
     const int nw = wd.w_hi - wd.w_lo;
+    if constexpr (kPool) {
+      const int nw8 = (nw + 7) & ~7;
+      by = reinterpret_cast<unsigned short*>(bx + nw8);
+      acc = reinterpret_cast<Acc*>(by + nw8);
+      cnt = min(cnt, (kWinPool - 6 * nw8) / (int)sizeof(Acc));  // holds by the cut
+    }
     if (hbits) {
       const unsigned* src = hbits + (size_t)((int64_t)wd.h * spans + wd.span) * kSpanWords + wd.w_lo;
       for (int w = tid; w < nw; w += CTA) bx[w] = kStreamOut ? __ldcs(src + w) : src[w];
@@ -411,7 +430,7 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
     }
 
     if (!hbits) {  // pass 1: rebuild the window's columns
-      for_row_pieces<2>(A, B, i, lo, hi, whole, b_sorted != 0, sm, [](int64_t) { return 0; },
+      for_row_pieces<2>(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, [](int64_t) { return 0; },
                                [](int64_t) { return 0; }, [&](int, int c, int) {
                           const unsigned off = (unsigned)((int64_t)c - lo);
                           const unsigned bit = 1u << (off & 31);
@@ -435,7 +454,7 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
     // pass 2: accumulate at the rank of each product's column (pieces of
     // 128 products of one B row per warp, loads first, then the atomics)
     const unsigned lo32 = (unsigned)lo;
-    for_row_pieces<4>(A, B, i, lo, hi, whole, b_sorted != 0, sm,
+    for_row_pieces<4>(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm,
                       [&](int64_t q) { return ldg_val(Bval + q); },
                       [&](int64_t p) { return S::kUsesA ? ldg_val(Aval + p) : TA(); },
                       [&](TA a_cur, int c, TB bv) {
@@ -471,10 +490,15 @@ __global__ void __launch_bounds__(CTA, CTA == 512 ? 3 : 1) k_num_rank(DevCSR A, 
         if (guard(out + t < row_end, 38, out + t))
           st_out(Cval + out + t, S::out(kL2 ? __ldcg(wacc + t) : wacc[t]));
     }
-    for_bitmap_columns<kL2 ? kDenseWordBits : 0, CTA>(bx, by, nw, cnt, [&](int j, int c) {
-      const int64_t o = out + j;
-      if (guard(o < row_end, 39, o)) st_out(Ccol + o, (int32_t)(lo + c));
-    });
+    if constexpr (kPool) {  // the accumulators are free once the values are out
+      __syncthreads();
+      write_columns<CTA>(bx, by, nw, cnt, row_end - out, (int32_t)lo, reinterpret_cast<int32_t*>(acc), Ccol + out);
+    } else {
+      for_bitmap_columns<kL2 ? kDenseWordBits : 0, CTA>(bx, by, nw, cnt, [&](int j, int c) {
+        const int64_t o = out + j;
+        if (guard(o < row_end, 39, o)) st_out(Ccol + o, (int32_t)(lo + c));
+      });
+    }
     take_unit(queue, &next);
     __syncthreads();
   }
@@ -496,7 +520,7 @@ void numeric_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, const int
                 const int32_t* heavy_rows, const Window* wins, int64_t n_wins,
                 const int32_t* span_counts, int64_t spans, const unsigned* hbits, int b_sorted,
                 const int64_t* Crp, int32_t* Ccol, void* Cval_, int64_t* counters, cudaStream_t s,
-                int sms, int* launches, int64_t num_hash_max, void* racc, CfBounds cf) {
+                int sms, int* launches, int64_t num_hash_max, void* racc, CfBounds cf, const SplitTable& tab) {
   typedef typename Sem<SR>::A Acc;
   typedef typename Sem<SR>::TC TC;
   TC* Cval = reinterpret_cast<TC*>(Cval_);
@@ -528,14 +552,12 @@ void numeric_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, const int
     ++*launches;
   }
   if (n_wins) {
-    // windows whose accumulators take little or no shared memory run three
-    // 512-thread CTAs per SM, three windows at once (RankShape)
     constexpr int CTA = RankShape<SR>::kCta;
-    constexpr int PER_SM = CTA == 512 ? 3 : 1;
+    constexpr int PER_SM = RankShape<SR>::kPerSm;
     constexpr size_t smem = RankShape<SR>::kSmem;
     set_smem(k_num_rank<SR, CTA>, smem);
     k_num_rank<SR, CTA><<<capped(n_wins, (int64_t)sms * PER_SM), CTA, smem, s>>>(
-        A, B, heavy_rows, wins, n_wins, span_counts, spans, hbits, b_sorted, flops, nnz, Crp, Ccol,
+        A, B, tab, heavy_rows, wins, n_wins, span_counts, spans, hbits, b_sorted, flops, nnz, Crp, Ccol,
         Cval, err, counters + kNumQueue, num_hash_max, static_cast<Acc*>(racc));
     ++*launches;
   }
@@ -573,10 +595,10 @@ void numeric_dev_sr(const DevCSR& A, const DevCSR& B, const int32_t* perm, int64
   }
   {  // rank windows of the heavy rows (window count read on the device)
     constexpr int CTA = RankShape<SR>::kCta;
-    constexpr int PER_SM = CTA == 512 ? 3 : 1;
+    constexpr int PER_SM = RankShape<SR>::kPerSm;
     constexpr size_t smem = RankShape<SR>::kSmem;
     k_num_rank<SR, CTA><<<sms * PER_SM, CTA, smem, s>>>(
-        A, B, perm_sym, wins, 0, span_counts, spans, nullptr, 0, flops, nnz, Crp, Ccol, Cval, err,
+        A, B, SplitTable{}, perm_sym, wins, 0, span_counts, spans, nullptr, 0, flops, nnz, Crp, Ccol, Cval, err,
         counters + kNumQueue, num_hash_max, static_cast<Acc*>(racc), counters);
   }
 }
@@ -643,12 +665,12 @@ int learn_hash_max(int sr) {
   }
 }
 
-int num_window_cut(int sr) {
+WinCut num_window_cut(int sr) {
   switch (sr) {
-#define CB_CASE(SRV) case SRV: return NumLimits<SRV>::kWcut;
+#define CB_CASE(SRV) case SRV: return RankShape<SRV>::kCut;
     CB_FOR_EACH_SEMIRING(CB_CASE)
 #undef CB_CASE
-    default: return 0;
+    default: return WinCut{};
   }
 }
 
@@ -667,11 +689,11 @@ void launch_numeric(int sr, const DevCSR& A, const DevCSR& B, const int32_t* per
                     int64_t n_wins, const int32_t* span_counts, int64_t spans,
                     const unsigned* hbits, int b_sorted, const int64_t* Crp, int32_t* Ccol,
                     void* Cval, int64_t* counters, cudaStream_t s, int sms, int* launches,
-                    int64_t num_hash_max, void* racc, CfBounds cf) {
+                    int64_t num_hash_max, void* racc, CfBounds cf, const SplitTable& tab) {
 #define CB_NUM(SRV)                                                                        \
   numeric_sr<SRV>(A, B, perm, seg_begin, seg_count, flops, nnz, heavy_rows, wins, n_wins,   \
                   span_counts, spans, hbits, b_sorted, Crp, Ccol, Cval, counters, s, sms, launches, \
-                  num_hash_max, racc, cf)
+                  num_hash_max, racc, cf, tab)
   switch (sr) {
 #define CB_CASE(SRV) case SRV: CB_NUM(SRV); break;
     CB_FOR_EACH_SEMIRING(CB_CASE)

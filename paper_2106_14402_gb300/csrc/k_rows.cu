@@ -149,6 +149,29 @@ __global__ void __launch_bounds__(256) k_tier_scatter(int64_t m, TierBySize tier
   else if (t > 0) perm[base[t] + slot] = (int32_t)i;
 }
 
+// Split table of a sorted B: one warp per row, a lane per boundary.  Rank
+// windows look a row's crossing up here and search only the entries between
+// two boundaries (a row of 2000 entries over 2^18 columns: 31 entries on four
+// sectors instead of eleven probes all over the row).  R-MAT s18 numeric: f64
+// 47.5 -> 46.2 ms, u32 36.8 -> 34.0, the table (68 MB) included.  Boundaries
+// lie 2^kSplitShift columns apart, further where the table would exceed
+// kSplitMaxBytes.
+constexpr int kSplitShift = 12;
+constexpr int64_t kSplitMaxBytes = int64_t(256) << 20;
+__global__ void __launch_bounds__(256) k_split_table(DevCSR B, int stride, int shift, int32_t* pos) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
+  for (int64_t k = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); k < B.nrows; k += nwarps) {
+    const int64_t q0 = B.rp[k], q1 = row_end(B, k);
+    for (int g = lane; g < stride; g += 32) {
+      const int64_t q = g == 0            ? q0
+                        : g == stride - 1 ? q1
+                                          : seq_lower_bound(B.col, q0, q1, B.col_lo + ((int64_t)g << shift));
+      pos[k * stride + g] = (int32_t)(q - q0);
+    }
+  }
+}
+
 // K4: three-pass exclusive scan (tile reduce, scan of tile sums, apply).
 constexpr int kScanThreads = 1024;
 constexpr int kScanItems = 4;
@@ -331,6 +354,23 @@ void launch_slabs(const DevCSR& B, const int64_t* bnd, int nb1, int64_t* pos, cu
                   int sms) {
   if (B.nrows == 0 || nb1 == 0) return;
   k_slabs<<<grid_for(B.nrows, 8, sms * 8), 256, 0, s>>>(B, bnd, nb1, pos);
+}
+
+SplitTable split_table_shape(int64_t n, int64_t ncols, size_t* bytes) {
+  SplitTable t;
+  *bytes = 0;
+  t.shift = kSplitShift;
+  if (ncols <= (int64_t(1) << t.shift)) return t;
+  const auto size = [&] { return ((ncols + (int64_t(1) << t.shift) - 1) >> t.shift) + 1; };
+  while (size() * n * 4 > kSplitMaxBytes && t.shift < 30) ++t.shift;
+  t.stride = (int)size();
+  *bytes = (size_t)t.stride * (size_t)n * 4;
+  return t;
+}
+
+void launch_split_table(const DevCSR& B, const SplitTable& t, cudaStream_t s, int sms) {
+  if (B.nrows == 0 || !t.stride) return;
+  k_split_table<<<grid_for(B.nrows, 8, sms * 8), 256, 0, s>>>(B, t.stride, t.shift, const_cast<int32_t*>(t.pos));
 }
 
 void launch_classify_num(int, int64_t m, const int64_t* nnz, int32_t* perm, int64_t* counters,

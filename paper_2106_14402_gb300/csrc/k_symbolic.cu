@@ -74,11 +74,11 @@ __global__ void __launch_bounds__(CTA) k_sym_hash(DevCSR A, DevCSR B, const int3
 
 // Heavy rows (u > 512): one CTA per (heavy row h, span) unit.  The bitmap
 // covers the span's columns [lo, hi); after counting, the span is cut into
-// rank windows of at most wcut + 31 entries (see cb_common.cuh), appended to
+// rank windows (WinCut), appended to
 // `wins` (when non-null) for the numeric phase.  Units are taken from a queue.
 __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, const int32_t* heavy_rows,
                                                      int64_t n_heavy, int64_t spans,
-                                                     const int64_t* flops, int wcut, int64_t* nnz,
+                                                     const int64_t* flops, WinCut wcut, int64_t* nnz,
                                                      int32_t* span_counts, int2* span_wins,
                                                      Window* wins, int64_t win_cap,
                                                      unsigned* hbits, int b_sorted,
@@ -124,7 +124,7 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
     }
     const int nwords = (int)((hi - lo + 31) / 32);
     const unsigned lo32 = (unsigned)lo;
-    for_row_pieces<4>(A, B, i, lo, hi, spans == 1 && !B.filter, b_sorted != 0, sm,
+    for_row_pieces<4>(A, B, SplitTable{}, i, lo, hi, spans == 1 && !B.filter, b_sorted != 0, sm,
                              [](int64_t) { return 0; }, [](int64_t) { return 0; }, [&](int, int c, int) {
                         const unsigned off = (unsigned)c - lo32;
                         const unsigned bit = 1u << (off & 31);
@@ -144,13 +144,13 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
     for (int j = 0; j < WPT; ++j) mine += c[j];
     int total;
     int run = team_exclusive_scan<1024>(mine, scratch, total);  // entries before my first word
-    // Windows: word w belongs to window floor(before(w) / wcut), where
-    // before(w) counts the entries in words < w.  Consecutive words differ by
-    // at most 32 <= wcut entries, so window indices run 0..K-1 without gaps,
-    // every window has a first word, and each holds at most wcut + 31 entries.
-    const int last_before = total - __popc(sym_bm[nwords - 1]);
-    int K = (wins && total > 0) ? last_before / wcut + 1 : 0;
-    if (K > kMaxWindowsPerSpan) {  // wcut too small for this span width
+    // Windows: word w belongs to window floor(weight(w) / cut), where
+    // weight(w) = per_word * w + per_entry * (entries in words < w).  A word
+    // adds at most per_word + 32 * per_entry <= cut, so window indices run
+    // 0..K-1 without gaps and every window has a first word.
+    const int last = wcut.per_word * (nwords - 1) + wcut.per_entry * (total - __popc(sym_bm[nwords - 1]));
+    int K = (wins && total > 0) ? last / wcut.cut + 1 : 0;
+    if (K > kMaxWindowsPerSpan) {  // cut too small for this span width
       if (tid == 0) atomicCAS((unsigned long long*)&counters[kError], 0ull, 31ull);
       K = 0;
     }
@@ -159,25 +159,27 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
       wrank[0] = 0;
     }
     // kcur = the window of the word before the current one; one division
-    // per thread, then a comparison per word (a word adds at most 32 <= wcut
-    // entries, so it crosses at most one multiple of wcut)
-    int kcur = 0, nextb = wcut;
+    // per thread, then a comparison per word (a word crosses at most one
+    // multiple of cut)
+    int weight = wcut.per_word * tid * WPT + wcut.per_entry * run;
+    int kcur = 0, nextb = wcut.cut;
     if (tid * WPT > 0 && tid * WPT < nwords) {
-      kcur = (run - __popc(sym_bm[tid * WPT - 1])) / wcut;
-      nextb = (kcur + 1) * wcut;
+      kcur = (weight - wcut.per_word - wcut.per_entry * __popc(sym_bm[tid * WPT - 1])) / wcut.cut;
+      nextb = (kcur + 1) * wcut.cut;
     }
 #pragma unroll
     for (int j = 0; j < WPT; ++j) {
       const int w = tid * WPT + j;
-      if (w > 0 && w < nwords && run >= nextb) {  // word w opens window kcur + 1
+      if (w > 0 && w < nwords && weight >= nextb) {  // word w opens window kcur + 1
         ++kcur;
-        nextb += wcut;
+        nextb += wcut.cut;
         if (kcur < K) {
           wstart[kcur] = w;
           wrank[kcur] = run;
         }
       }
       run += c[j];
+      weight += wcut.per_word + wcut.per_entry * c[j];
     }
     if (tid == 0) {
       long long b = -1;
@@ -254,7 +256,7 @@ void prepare_symbolic_dev() {
 
 void launch_symbolic_dev(const DevCSR& A, const DevCSR& B, const int32_t* perm, int64_t* counters,
                          const int64_t* flops, int64_t* nnz, int32_t* span_counts, int2* span_wins,
-                         int wcut, Window* wins, int64_t win_cap, cudaStream_t s, int sms) {
+                         WinCut wcut, Window* wins, int64_t win_cap, cudaStream_t s, int sms) {
   const int64_t m = A.nrows;
   if (m == 0) return;
   {  // heavy rows (bitmaps, rank windows), count and B's sortedness read on the device
@@ -287,7 +289,7 @@ void launch_symbolic_dev(const DevCSR& A, const DevCSR& B, const int32_t* perm, 
 
 void launch_symbolic(const DevCSR& A, const DevCSR& B, const int32_t* perm,
                      const int64_t* seg_begin, const int64_t* seg_count, const int64_t* flops,
-                     int64_t* nnz, int32_t* span_counts, int2* span_wins, int wcut,
+                     int64_t* nnz, int32_t* span_counts, int2* span_wins, WinCut wcut,
                      Window* wins, int64_t win_cap, unsigned* hbits, int b_sorted,
                      int64_t* counters, cudaStream_t s, int sms, int* launches) {
   if (seg_count[kSymWarp]) {
