@@ -699,249 +699,105 @@ __device__ __forceinline__ void row_slice(const DevCSR& B, const SplitTable& t, 
   s1 = b0;
 }
 
-// Shared memory used by for_row_products_balanced: per chunk entry with a
-// nonempty product range, its product offset, its first B index and its A
-// index (relative to the chunk), plus scan scratch.
-struct BalancedSmem {
-  long long* off;  // [blockDim.x]
-  long long* b0;   // [blockDim.x]
-  int* pa;         // [blockDim.x]
-  long long* scan; // [33]
-  int* iscan;      // [33]
-};
+// Marks a call of for_row_pieces that needs no values of B.
+struct NoValue {};
 
-// Load-balanced form of for_row_products for a whole CTA: the row's stored
-// A entries are taken in chunks of blockDim.x; the chunk's nonempty product
-// ranges (B row, or the B row's slice in [lo, hi) when `sorted` and not
-// `whole`) are compacted and prefix-summed, every warp takes an equal
-// contiguous share of the chunk's products and its lanes take consecutive
-// products (coalesced B reads).  Short ranges (< kLongRange products) and
-// long ones are done in two rounds:
-//   * short: since ranges are nonempty, the 32 products of one warp step
-//     start at most 31 new ranges: each lane reads one range start, the warp
-//     ORs together the bits of the starts that fall inside the step, and a
-//     lane's range is the step's first range plus the number of starts at or
-//     before its product;
-//   * long: the warp walks its share range by range, 32 * U consecutive
-//     products of one range per iteration, with no per-product range
-//     bookkeeping (the A entry is uniform over the warp).
-// All threads of the CTA must call it.
-constexpr int kLongRange = 128;
-constexpr int kLongUnroll = 2;   // warp steps per iteration of the long round, in units of U
-
-template <int U, class LD, class F>
-__device__ __forceinline__ void for_row_products_balanced_u(const DevCSR& A, const DevCSR& B,
-                                                            int64_t i, int64_t lo, int64_t hi,
-                                                            bool whole, bool sorted,
-                                                            const BalancedSmem& sm, LD&& ld, F&& f) {
-  typedef decltype(ld(int64_t(0))) V;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int nthr = blockDim.x, nwarp = nthr >> 5;
-  const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
-  const bool filter = !whole && !sorted;
-  const unsigned width = (unsigned)(hi - lo);
-  for (int64_t c0 = a0; c0 < a1; c0 += nthr) {
-    const int nch = (int)min((int64_t)nthr, a1 - c0);
-    long long len = 0;
-    int64_t q0 = 0;
-    if (tid < nch) {
-      const int k = A.col[c0 + tid];
-      q0 = B.rp[k];
-      int64_t q1 = row_end(B, k);
-      if (!whole && sorted) {
-        const int64_t s0 = seq_lower_bound(B.col, q0, q1, lo);
-        q1 = seq_lower_bound(B.col, s0, q1, hi);
-        q0 = s0;
-      }
-      len = q1 - q0;
-    }
-    // a round with no ranges of its kind in the chunk is skipped (uniform)
-    const int any_short = __syncthreads_or(len > 0 && len < kLongRange);
-    const int any_long = __syncthreads_or(len >= kLongRange);
-    for (int round = 0; round < 2; ++round) {
-      if (!(round == 0 ? any_short : any_long)) continue;
-      const long long lr = (round == 0) == (len < kLongRange) ? len : 0;
-      // one scan gives both the product offsets (high bits) and the slots of
-      // the nonempty ranges (low 11 bits; at most 1024 of them)
-      long long packed_total;
-      const long long packed =
-          cta_exclusive_scan64((lr << 11) | (lr > 0 ? 1 : 0), sm.scan, packed_total);
-      const long long total = packed_total >> 11;
-      const int ne = (int)(packed_total & 2047);
-      if (lr > 0) {
-        const int slot = (int)(packed & 2047);
-        sm.off[slot] = packed >> 11;
-        sm.b0[slot] = q0;
-        sm.pa[slot] = tid;
-      }
-      __syncthreads();
-      const long long t_beg = total * warp / nwarp, t_end = total * (warp + 1) / nwarp;
-      if (round == 1 && t_beg < t_end) {
-        // range holding the warp's first product
-        int l = 0, r = ne - 1;
-        while (l < r) {
-          const int mid = (l + r + 1) >> 1;
-          if (sm.off[mid] <= t_beg) l = mid;
-          else r = mid - 1;
-        }
-        int j = l;
-        constexpr int UL = U * kLongUnroll;
-        for (long long t = t_beg; t < t_end; ++j) {  // uniform over the warp
-          const long long r_end = j + 1 < ne ? sm.off[j + 1] : total;
-          const long long e = r_end < t_end ? r_end : t_end;
-          const int64_t qb = sm.b0[j] - sm.off[j];
-          const int64_t pc = c0 + sm.pa[j];
-          for (long long tt = t; tt < e; tt += 32 * UL) {
-            int64_t qu[UL];
-            bool vu[UL];
-#pragma unroll
-            for (int u = 0; u < UL; ++u) {
-              const long long x = tt + 32 * u + lane;
-              vu[u] = x < e;
-              qu[u] = qb + x;
-            }
-            int cu[UL];
-            V vv[UL];
-#pragma unroll
-            for (int u = 0; u < UL; ++u) {
-              cu[u] = vu[u] ? __ldg(B.col + qu[u]) : 0;
-              vv[u] = vu[u] ? ld(qu[u]) : V();
-            }
-#pragma unroll
-            for (int u = 0; u < UL; ++u)
-              if (vu[u] && (!filter || (unsigned)((int64_t)cu[u] - lo) < width)) f(pc, qu[u], cu[u], vv[u]);
-          }
-          t = e;
-        }
-      }
-      if (round == 0 && t_beg < t_end) {
-        // range holding the warp's first product (the same search in every lane)
-        int l = 0, r = ne - 1;
-        while (l < r) {
-          const int mid = (l + r + 1) >> 1;
-          if (sm.off[mid] <= t_beg) l = mid;
-          else r = mid - 1;
-        }
-        int j0 = l;
-        long long nxt = j0 + 1 < ne ? sm.off[j0 + 1] : LLONG_MAX;  // start of the next range
-        int jc = -1;          // the lane's current range, its B offset and A entry
-        int64_t qb = 0, pc = 0;
-        // U warp steps per iteration: positions first, then all loads, then
-        // the callbacks, so that U independent loads are in flight per lane
-        for (long long tb = t_beg; tb < t_end; tb += 32 * U) {
-          int64_t qu[U], pu[U];
-          bool vu[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            const long long ts = tb + 32 * u;
-            int j = j0;
-            if (nxt <= ts + 31) {  // the step crosses range starts (uniform over the warp)
-              const int k = j0 + 1 + lane;
-              const long long st = k < ne ? sm.off[k] : LLONG_MAX;
-              const long long pos = st - ts;  // >= 1 by the choice of j0
-              const unsigned bits = __reduce_or_sync(0xffffffffu, pos < 32 ? 1u << (int)pos : 0u);
-              j = j0 + __popc(bits & ((2u << lane) - 1u));
-              j0 += __popc(bits);
-              nxt = j0 + 1 < ne ? sm.off[j0 + 1] : LLONG_MAX;
-            }
-            const long long t = ts + lane;
-            vu[u] = t < t_end;
-            if (vu[u] && j != jc) {
-              jc = j;
-              qb = sm.b0[j] - sm.off[j];
-              pc = c0 + sm.pa[j];
-            }
-            qu[u] = qb + t;
-            pu[u] = pc;
-            // range holding product ts + 32 (ranges are nonempty, so at most one more start)
-            if (nxt <= ts + 32) {
-              ++j0;
-              nxt = j0 + 1 < ne ? sm.off[j0 + 1] : LLONG_MAX;
-            }
-          }
-          int cu[U];
-          V vv[U];
-#pragma unroll
-          for (int u = 0; u < U; ++u) {
-            cu[u] = vu[u] ? __ldg(B.col + qu[u]) : 0;
-            vv[u] = vu[u] ? ld(qu[u]) : V();
-          }
-#pragma unroll
-          for (int u = 0; u < U; ++u)
-            if (vu[u] && (!filter || (unsigned)((int64_t)cu[u] - lo) < width)) f(pu[u], qu[u], cu[u], vv[u]);
-        }
-      }
-      __syncthreads();
-    }
-  }
-}
-
-// Piece-wise form for a whole CTA: the row's stored A entries are taken in
-// chunks of blockDim.x; each entry's product range (its B row, or the B
-// row's slice in [lo, hi) when `sorted` and not `whole`) is cut into pieces
-// of at most 32 * U consecutive products, the chunk's pieces are numbered
-// by one CTA scan, and every warp takes an equal contiguous run of pieces.
-// Inside a piece the A entry is the same for the whole warp and lane l
-// takes products l, l + 32, ...: no per-product bookkeeping, coalesced B
-// reads, all loads of a piece in flight before the callbacks.
+// All products of row i whose columns lie in [lo, hi), for a whole CTA: the
+// row's stored A entries are taken in chunks of blockDim.x; each entry's
+// product range (its B row, or the B row's slice in [lo, hi) when `sorted` and
+// not `whole`) is cut into pieces of 128 consecutive entries of B, the chunk's
+// pieces are numbered by one CTA scan, and every warp takes an equal
+// contiguous run of pieces.  Inside a piece the A entry is the same for the
+// whole warp.
 //   on_entry(p): called (warp-uniformly) when the warp reaches the pieces of
 //                A entry p; returns a token (e.g. A's value) for them;
-//   f(t, c, v):  one product: the token, column c and the value ld(q) of its
-//                B entry.
+//   f(t, c, v):  one product: the token, column c and B's value there (values
+//                from Bval; V = NoValue reads none).
+// Lane l takes entries l, l + 32, l + 64, l + 96 of a piece: coalesced loads,
+// all in flight before the callbacks, and neighbouring lanes meet neighbouring
+// columns, whose accumulators often share an L2 sector (with four consecutive
+// entries per lane, read in 16-byte loads, fp64 numeric took 55 instead of 46
+// ms on R-MAT s18 and 21.7 instead of 14.9 on the block-clustered product).
+// The loop is bound by the instructions it issues, so a range's pieces are
+// walked in an inner loop on 32-bit offsets from its first entry.
 // All threads of the CTA must call it.
-// Whether full pieces take a path without per-product bounds checks.
-constexpr bool kFullPieces = true;
-
 struct PieceSmem {
   int* poff;        // [blockDim.x] first piece of each nonempty range (chunk numbering)
-  long long* q0;    // [blockDim.x] first B index of the range
-  long long* len;   // [blockDim.x] products in the range
+  long long* q0;    // [blockDim.x] first B entry of the range
+  int* len;         // [blockDim.x] entries in the range
   int* pa;          // [blockDim.x] A entry of the range (relative to the chunk)
   long long* scan;  // [33]
-  static constexpr size_t kBytesPerThread = sizeof(int) + 2 * sizeof(long long) + sizeof(int);
+  static constexpr size_t kBytesPerThread = sizeof(long long) + 3 * sizeof(int);
+  // carved from threads * kBytesPerThread bytes, 8-byte aligned
+  __device__ PieceSmem(void* p, int threads, long long* scan_) : scan(scan_) {
+    q0 = static_cast<long long*>(p);
+    len = reinterpret_cast<int*>(q0 + threads);
+    poff = len + threads;
+    pa = poff + threads;
+  }
 };
 
-template <int U, class LD, class FA, class F>
+template <class V, class FA, class F>
 __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B, const SplitTable& tab,
                                                int64_t i, int64_t lo, int64_t hi, bool whole, bool sorted,
-                                               const PieceSmem& sm, LD&& ld, FA&& on_entry, F&& f) {
-  typedef decltype(ld(int64_t(0))) V;
-  typedef decltype(on_entry(int64_t(0))) T;
-  constexpr int P = 32 * U;
+                                               const PieceSmem& sm, const V* Bval, FA&& on_entry, F&& f) {
+  constexpr int P = 128;
+  constexpr bool kVals = !std::is_same<V, NoValue>::value;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nthr = blockDim.x, nwarp = nthr >> 5;
   const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
   const bool filter = !whole && !sorted;
   const unsigned width = (unsigned)(hi - lo);
+  const unsigned lo32 = (unsigned)lo;
   for (int64_t c0 = a0; c0 < a1; c0 += nthr) {
     const int nch = (int)min((int64_t)nthr, a1 - c0);
-    long long len = 0;
-    int64_t q0 = 0;
+    int64_t q0 = 0, q1 = 0;
     if (tid < nch) {
       const int k = A.col[c0 + tid];
-      q0 = B.rp[k];
-      int64_t q1 = row_end(B, k);
-      if (!whole && sorted) row_slice(B, tab, k, lo, hi, q0, q1);
-      len = q1 - q0;
+      if (!whole && sorted) {
+        row_slice(B, tab, k, lo, hi, q0, q1);
+      } else {
+        q0 = B.rp[k];
+        q1 = row_end(B, k);
+      }
     }
-    const long long np = (len + P - 1) / P;
+    const long long np = q0 < q1 ? (q1 - q0 + P - 1) / P : 0;
     // one scan numbers the pieces (high bits) and the nonempty ranges (low 11 bits)
     long long packed_total;
     const long long packed = cta_exclusive_scan64((np << 11) | (np > 0 ? 1 : 0), sm.scan, packed_total);
     const long long npieces = packed_total >> 11;
     const int ne = (int)(packed_total & 2047);
+    if (npieces >= (1 << 24)) {  // 2^31 products or more: 32-bit offsets do not do; entry by entry
+      for (int t = 0; t < nch; ++t) {
+        if (tid == t) {
+          sm.q0[0] = q0;
+          sm.q0[1] = q1;
+        }
+        __syncthreads();
+        const auto tok = on_entry(c0 + t);
+        const int64_t end = sm.q0[1];
+        for (int64_t q = sm.q0[0] + tid; q < end; q += nthr) {
+          const int c = __ldg(B.col + q);
+          V v{};
+          if constexpr (kVals) v = ldg_val(Bval + q);
+          if (!filter || (unsigned)c - lo32 < width) f(tok, c, v);
+        }
+        __syncthreads();
+      }
+      continue;
+    }
     if (np > 0) {
       const int slot = (int)(packed & 2047);
       sm.poff[slot] = (int)(packed >> 11);
       sm.q0[slot] = q0;
-      sm.len[slot] = len;
+      sm.len[slot] = (int)(q1 - q0);
       sm.pa[slot] = tid;
     }
     __syncthreads();
     // equal runs of pieces per warp; nwarp is a power of two (512- and
     // 1024-thread CTAs), so the split needs no 64-bit division
     const int lgw = 31 - __clz(nwarp);
-    const long long k_beg = (npieces * warp) >> lgw, k_end = (npieces * (warp + 1)) >> lgw;
+    const int k_beg = (int)((npieces * warp) >> lgw), k_end = (int)((npieces * (warp + 1)) >> lgw);
     if (k_beg < k_end) {  // uniform over the warp
       int l = 0, r = ne - 1;  // range holding piece k_beg
       while (l < r) {
@@ -949,84 +805,40 @@ __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B,
         if (sm.poff[mid] <= k_beg) l = mid;
         else r = mid - 1;
       }
-      int j = l;
-      long long pj = sm.poff[j];
-      long long nxt = j + 1 < ne ? sm.poff[j + 1] : LLONG_MAX;
-      int64_t qj = sm.q0[j];
-      long long lj = sm.len[j];
-      T tok = on_entry(c0 + sm.pa[j]);
-      // one piece: its products' columns and values in registers
-      struct Piece {
-        int n;
-        T tok;
-        int c[U];
-        V v[U];
-      };
-      const auto load = [&](long long k, Piece& pc) {
-        if (k >= nxt) {  // the next range starts here (ranges are nonempty)
-          ++j;
-          pj = nxt;
-          nxt = j + 1 < ne ? sm.poff[j + 1] : LLONG_MAX;
-          qj = sm.q0[j];
-          lj = sm.len[j];
-          tok = on_entry(c0 + sm.pa[j]);
-        }
-        const long long s0 = (k - pj) * P;
-        pc.n = (int)min((long long)P, lj - s0);
-        pc.tok = tok;
-        const int64_t qs = qj + s0;
-        const int32_t* cp = B.col + qs;
-        if (kFullPieces && pc.n == P) {  // a full piece: no bounds to check (uniform)
+      int s = (k_beg - sm.poff[l]) * P;  // first entry of the next piece
+      for (int j = l, left = k_end - k_beg; left > 0; ++j, s = 0) {
+        const int len = sm.len[j];
+        const int32_t* cp = B.col + sm.q0[j] + lane;
+        const V* vp = kVals ? Bval + sm.q0[j] + lane : nullptr;
+        const auto tok = on_entry(c0 + sm.pa[j]);
+        for (; left > 0 && s < len; --left, s += P) {
+          int c[4];
+          V v[4];
+          if (s + P <= len && !filter) {  // a whole piece (uniform)
 #pragma unroll
-          for (int u = 0; u < U; ++u) {
-            pc.c[u] = __ldg(cp + u * 32 + lane);
-            pc.v[u] = ld(qs + u * 32 + lane);
-          }
-          return;
-        }
+            for (int u = 0; u < 4; ++u) {
+              c[u] = __ldg(cp + s + 32 * u);
+              if constexpr (kVals) v[u] = ldg_val(vp + s + 32 * u);
+            }
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int x = u * 32 + lane;
-          pc.c[u] = 0;
-          pc.v[u] = V();
-          if (u * 32 < pc.n && x < pc.n) {
-            pc.c[u] = __ldg(cp + x);
-            pc.v[u] = ld(qs + x);
+            for (int u = 0; u < 4; ++u) f(tok, c[u], v[u]);
+          } else {
+            const int n = len - s - lane;  // the lane's entries: 32 * u < n
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (32 * u < n) {
+                c[u] = __ldg(cp + s + 32 * u);
+                if constexpr (kVals) v[u] = ldg_val(vp + s + 32 * u);
+              }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+              if (32 * u < n && (!filter || (unsigned)c[u] - lo32 < width)) f(tok, c[u], v[u]);
           }
         }
-      };
-      const auto consume = [&](const Piece& pc) {
-        if (kFullPieces && pc.n == P && !filter) {
-#pragma unroll
-          for (int u = 0; u < U; ++u) f(pc.tok, pc.c[u], pc.v[u]);
-          return;
-        }
-#pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int x = u * 32 + lane;
-          if (u * 32 < pc.n && x < pc.n && (!filter || (unsigned)((int64_t)pc.c[u] - lo) < width))
-            f(pc.tok, pc.c[u], pc.v[u]);
-        }
-      };
-      for (long long k = k_beg; k < k_end; ++k) {
-        Piece cur;
-        load(k, cur);
-        consume(cur);
       }
     }
     __syncthreads();
   }
-}
-
-// The loop above with one warp step per iteration and no value loads.
-template <class F>
-__device__ __forceinline__ void for_row_products_balanced(const DevCSR& A, const DevCSR& B,
-                                                          int64_t i, int64_t lo, int64_t hi,
-                                                          bool whole, bool sorted,
-                                                          const BalancedSmem& sm, F&& f) {
-  for_row_products_balanced_u<1>(A, B, i, lo, hi, whole, sorted, sm,
-                                 [](int64_t) { return 0; },
-                                 [&](int64_t p, int64_t q, int c, int) { f(p, q, c); });
 }
 
 }  // namespace cb

@@ -361,8 +361,7 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
   long long* bal = reinterpret_cast<long long*>(rank_smem + RankShape<SR>::kAccBytes + RankShape<SR>::kWordBytes);
   __shared__ int scratch[33];
   __shared__ long long scan64[33];
-  const PieceSmem sm{reinterpret_cast<int*>(bal + 2 * CTA), bal, bal + CTA,
-                     reinterpret_cast<int*>(bal + 2 * CTA) + CTA, scan64};
+  const PieceSmem sm(bal, CTA, scan64);
   __shared__ long long s_base;
   __shared__ long long next;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -430,12 +429,11 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
     }
 
     if (!hbits) {  // pass 1: rebuild the window's columns
-      for_row_pieces<2>(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, [](int64_t) { return 0; },
-                               [](int64_t) { return 0; }, [&](int, int c, int) {
-                          const unsigned off = (unsigned)((int64_t)c - lo);
-                          const unsigned bit = 1u << (off & 31);
-                          if (chk(off < 32u * (unsigned)nw, 36, c)) atomicOr(&bx[off >> 5], bit);
-                        });
+      for_row_pieces(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, (const NoValue*)nullptr,
+                     [](int64_t) { return 0; }, [&](int, int c, NoValue) {
+                       const unsigned off = (unsigned)((int64_t)c - lo);
+                       if (chk(off < 32u * (unsigned)nw, 36, c)) atomicOr(&bx[off >> 5], 1u << (off & 31));
+                     });
       __syncthreads();
     }
     // exclusive prefix of word popcounts
@@ -451,27 +449,25 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
       if (tid == 0 && total != wd.count) flag_error(err, 23);
     }
     __syncthreads();
-    // pass 2: accumulate at the rank of each product's column (pieces of
-    // 128 products of one B row per warp, loads first, then the atomics)
+    // pass 2: accumulate at the rank of each product's column: the entries of
+    // the words before its word and the word's bits up to it, less itself
     const unsigned lo32 = (unsigned)lo;
-    for_row_pieces<4>(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm,
-                      [&](int64_t q) { return ldg_val(Bval + q); },
-                      [&](int64_t p) { return S::kUsesA ? ldg_val(Aval + p) : TA(); },
-                      [&](TA a_cur, int c, TB bv) {
-                        const unsigned off = (unsigned)c - lo32;
-                        if (!chk(off < 32u * (unsigned)nw, 36, c)) return;
-                        const uint2 e = make_uint2(bx[off >> 5], by[off >> 5]);
-                        const int slot = (int)e.y + __popc(e.x & ((1u << (off & 31)) - 1u));
-                        if (guard(slot < lim, 37, out + slot)) {
-                          if constexpr (kInPlace) {
-                            red_add_hint(&wacc[slot], S::mul(a_cur, bv), pol);
-                          } else if constexpr (kBits) {
-                            if (S::mul(a_cur, bv)) atomicOr(&accbits[slot >> 5], 1u << (slot & 31));
-                          } else {
-                            S::atomic(&wacc[slot], S::mul(a_cur, bv));
-                          }
-                        }
-                      });
+    for_row_pieces(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, Bval,
+                   [&](int64_t p) { return S::kUsesA ? ldg_val(Aval + p) : TA(); },
+                   [&](TA a_cur, int c, TB bv) {
+                     const unsigned off = (unsigned)c - lo32;
+                     if (!chk(off < 32u * (unsigned)nw, 36, c)) return;
+                     const int slot = (int)by[off >> 5] + __popc(bx[off >> 5] << (~off & 31u)) - 1;
+                     if (guard((unsigned)slot < (unsigned)lim, 37, out + slot)) {
+                       if constexpr (kInPlace) {
+                         red_add_hint(&wacc[slot], S::mul(a_cur, bv), pol);
+                       } else if constexpr (kBits) {
+                         if (S::mul(a_cur, bv)) atomicOr(&accbits[slot >> 5], 1u << (slot & 31));
+                       } else {
+                         S::atomic(&wacc[slot], S::mul(a_cur, bv));
+                       }
+                     }
+                   });
     __syncthreads();
     if (kInPlace && lim > 0) {  // the window is complete: its lines back to normal priority
       const uintptr_t b0 = reinterpret_cast<uintptr_t>(wacc) & ~(uintptr_t)127;

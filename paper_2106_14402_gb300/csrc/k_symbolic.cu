@@ -100,8 +100,7 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
   const int64_t units = n_heavy * spans;
   const int bm_words = (int)min((int64_t)kSpanWords, (B.ncols + 31) / 32);
   long long* bal = reinterpret_cast<long long*>(sym_bm + ((bm_words + 3) & ~3));
-  const PieceSmem sm{reinterpret_cast<int*>(bal + 2048), bal, bal + 1024,
-                     reinterpret_cast<int*>(bal + 2048) + 1024, scan64};
+  const PieceSmem sm(bal, 1024, scan64);
   // the bitmap starts clear; each unit clears the words it set once it has
   // read them, so no unit starts with a clearing pass of its own
   for (int w = tid; w < bm_words; w += 1024) sym_bm[w] = 0u;
@@ -124,12 +123,11 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
     }
     const int nwords = (int)((hi - lo + 31) / 32);
     const unsigned lo32 = (unsigned)lo;
-    for_row_pieces<4>(A, B, SplitTable{}, i, lo, hi, spans == 1 && !B.filter, b_sorted != 0, sm,
-                             [](int64_t) { return 0; }, [](int64_t) { return 0; }, [&](int, int c, int) {
-                        const unsigned off = (unsigned)c - lo32;
-                        const unsigned bit = 1u << (off & 31);
-                        if (chk(off < 32u * (unsigned)nwords, 40, c)) atomicOr(&sym_bm[off >> 5], bit);
-                      });
+    for_row_pieces(A, B, SplitTable{}, i, lo, hi, spans == 1 && !B.filter, b_sorted != 0, sm,
+                   (const NoValue*)nullptr, [](int64_t) { return 0; }, [&](int, int c, NoValue) {
+                     const unsigned off = (unsigned)c - lo32;
+                     if (chk(off < 32u * (unsigned)nwords, 40, c)) atomicOr(&sym_bm[off >> 5], 1u << (off & 31));
+                   });
     __syncthreads();
     if (hbits) {
       unsigned* dst = hbits + (size_t)(h * spans + sp) * kSpanWords;
