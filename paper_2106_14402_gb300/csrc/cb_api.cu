@@ -295,7 +295,7 @@ void check_words(cb_ctx* ctx) {
     int64_t (*take)(cudaStream_t, int64_t*);
   } const readers[] = {{"numeric", cb::check_take_numeric},   {"symbolic", cb::check_take_symbolic},
                        {"queue", cb::check_take_queue},       {"rows", cb::check_take_rows},
-                       {"fused", cb::check_take_fused}};
+                       {"fused", cb::check_take_fused},       {"pattern", cb::check_take_pattern}};
   for (const auto& r : readers) {
     int64_t index = 0;
     const int64_t code = r.take(ctx->stream, &index);
@@ -548,6 +548,11 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   CB_CUDA(cudaMemsetAsync(counters, 0, sizeof(int64_t) * cb::kCounters, ctx->stream));
   mark(ctx, opt, 0);
   cb::launch_check_sorted(dB, counters, ctx->stream, ctx->sms);
+  if (sr == CB_OR_AND_BOOL) {
+    cb::launch_any_false(dA, counters, ctx->stream, ctx->sms);
+    cb::launch_any_false(dB, counters, ctx->stream, ctx->sms);
+    ctx->stats.kernels += 2;
+  }
   cb::launch_classify_sym(dA, dB, flops, maxb, counters, ctx->stream, ctx->sms, skip,
                           ctx->tune.sym_hash_max);
   cb::launch_scatter_sym(m, ncols, flops, perm_sym, nnz, counters, ctx->stream, ctx->sms, skip,
@@ -557,6 +562,7 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   ctx->stats.kernels += 3;
   read_counters(ctx, counters, nullptr, 0);
   const int b_sorted = ctx->host[cb::kUnsorted] == 0 ? 1 : 0;
+  const bool all_true = sr == CB_OR_AND_BOOL && ctx->host[cb::kFalse] == 0;
 
   int64_t sym_cnt[cb::kSymTiers], sym_beg[cb::kSymTiers];
   for (int t = 0; t < cb::kSymTiers; ++t) sym_cnt[t] = ctx->host[cb::kCntSym + t];
@@ -689,13 +695,20 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   mark(ctx, opt, 4);
   // a pass over B's rows for the table pays once more than a few rows are cut
   // into several windows (a row's only window takes B's rows whole)
-  if (tab_pos && n_units > n_heavy + n_heavy / 8) {
+  if (tab_pos && !(all_true && hbits) && n_units > n_heavy + n_heavy / 8) {
     tab.pos = tab_pos;
     cb::launch_split_table(dB, tab, ctx->stream, ctx->sms);
     ++launches;
   }
+  // all true: rows with stored bitmaps are read out of them, leaving no windows
+  const bool pattern = all_true && hbits && n_units > 0;
+  if (pattern) {
+    cb::launch_pattern_rows(dA, dB, heavy_rows, n_heavy, spans, span_counts, hbits, nnz, C->row_ptr, C->col,
+                            C->val, counters, ctx->stream, ctx->sms, num_hash_max);
+    ++launches;
+  }
   cb::launch_numeric(sr, dA, dB, perm_num, num_beg, num_cnt, flops, nnz, heavy_rows, wins,
-                     n_units, span_counts, spans, hbits, b_sorted, C->row_ptr, C->col, C->val,
+                     pattern ? 0 : n_units, span_counts, spans, hbits, b_sorted, C->row_ptr, C->col, C->val,
                      counters, ctx->stream, ctx->sms, &launches, num_hash_max, racc,
                      cb::CfBounds{ctx->tune.cf_esc, ctx->tune.cf_pre}, tab);
   CB_LAUNCHED();

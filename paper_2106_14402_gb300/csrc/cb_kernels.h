@@ -85,7 +85,8 @@ enum Counter {
   kMaxArow = 26,        // longest row of A (k_classify_sym)
   kCurHeavy = 27,       // scatter cursor of the heavy rows placed from the segment's end
   kSymQueue = 28,       // next unit of the heavy rows' symbolic pass
-  kNumQueue = 29,       // next rank window of the numeric phase
+  kNumQueue = 29,       // next rank window (or span read out, k_pattern.cu) of the numeric phase
+  kFalse = 30,          // > 0 when a stored value of an (or,and) operand is false (k_any_false)
   kCounters = 32
 };
 
@@ -182,6 +183,15 @@ void launch_numeric(int sr, const DevCSR& A, const DevCSR& B, const int32_t* per
                     void* Cval, int64_t* counters, cudaStream_t s, int sms, int* launches,
                     int64_t num_hash_max = 512, void* racc = nullptr, CfBounds cf = {},
                     const SplitTable& tab = {});
+
+// (or,and) with no false value stored (k_pattern.cu): the check of one
+// operand (sets counters[kFalse]), and the numeric phase of the bitmap-tier
+// rows from their stored bitmaps alone.
+void launch_any_false(const DevCSR& M, int64_t* counters, cudaStream_t s, int sms);
+void launch_pattern_rows(const DevCSR& A, const DevCSR& B, const int32_t* heavy_rows, int64_t n_heavy,
+                         int64_t spans, const int32_t* span_counts, const unsigned* hbits, const int64_t* nnz,
+                         const int64_t* Crp, int32_t* Ccol, void* Cval, int64_t* counters, cudaStream_t s,
+                         int sms, int64_t num_hash_max);
 
 // Batched products (cb_batched.cu): stack parts into one CSR.
 size_t stack_part_size();
@@ -305,5 +315,6 @@ int64_t check_take_symbolic(cudaStream_t s, int64_t* index);
 int64_t check_take_queue(cudaStream_t s, int64_t* index);
 int64_t check_take_rows(cudaStream_t s, int64_t* index);
 int64_t check_take_fused(cudaStream_t s, int64_t* index);
+int64_t check_take_pattern(cudaStream_t s, int64_t* index);
 
 }  // namespace cb
