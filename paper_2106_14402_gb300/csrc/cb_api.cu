@@ -415,6 +415,7 @@ int queue_pass(cb_ctx* ctx, int sr, const DevCSR& dA, const DevCSR& dB, int64_t 
   ensure_fused(ctx, m);
   int* st = reinterpret_cast<int*>(ctx->fsync + 4);
   CB_CUDA(cudaMemsetAsync(st, 0, sizeof(int), ctx->stream));
+  CB_CUDA(cb::prepare_queue_rows(sr));
   mark(ctx, opt, 4);
   const cudaError_t e = cb::launch_queue_rows(sr, dA, dB, m, C->row_ptr, C->col, C->val, cap,
                                               ctx->fstat, ctx->fstat_cap, ctx->fsync, st, ctx->stream,
@@ -548,11 +549,6 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   CB_CUDA(cudaMemsetAsync(counters, 0, sizeof(int64_t) * cb::kCounters, ctx->stream));
   mark(ctx, opt, 0);
   cb::launch_check_sorted(dB, counters, ctx->stream, ctx->sms);
-  if (sr == CB_OR_AND_BOOL) {
-    cb::launch_any_false(dA, counters, ctx->stream, ctx->sms);
-    cb::launch_any_false(dB, counters, ctx->stream, ctx->sms);
-    ctx->stats.kernels += 2;
-  }
   cb::launch_classify_sym(dA, dB, flops, maxb, counters, ctx->stream, ctx->sms, skip,
                           ctx->tune.sym_hash_max);
   cb::launch_scatter_sym(m, ncols, flops, perm_sym, nnz, counters, ctx->stream, ctx->sms, skip,
@@ -562,7 +558,6 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   ctx->stats.kernels += 3;
   read_counters(ctx, counters, nullptr, 0);
   const int b_sorted = ctx->host[cb::kUnsorted] == 0 ? 1 : 0;
-  const bool all_true = sr == CB_OR_AND_BOOL && ctx->host[cb::kFalse] == 0;
 
   int64_t sym_cnt[cb::kSymTiers], sym_beg[cb::kSymTiers];
   for (int t = 0; t < cb::kSymTiers; ++t) sym_cnt[t] = ctx->host[cb::kCntSym + t];
@@ -639,6 +634,12 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   const int32_t* heavy_rows = perm_sym + sym_beg[cb::kSymHeavy];
 
   int launches = 0;
+  const bool check_true = sr == CB_OR_AND_BOOL && hbits;
+  if (check_true) {
+    cb::launch_any_false(dA, counters, ctx->stream, ctx->sms);
+    cb::launch_any_false(dB, counters, ctx->stream, ctx->sms);
+    launches += 2;
+  }
   cb::launch_symbolic(dA, dB, perm_sym, sym_beg, sym_cnt, flops, nnz, span_counts, span_wins, wcut,
                       wins, win_cap, hbits, b_sorted, counters, ctx->stream, ctx->sms, &launches);
   mark(ctx, opt, 2);
@@ -663,6 +664,8 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   num_beg[1] = 0;
   for (int t = 2; t < cb::kNumTiers; ++t) num_beg[t] = num_beg[t - 1] + num_cnt[t - 1];
   const int64_t n_units = ctx->host[cb::kUnits];
+  // all true: rows with stored bitmaps are read out of them, leaving no windows
+  const bool pattern = check_true && ctx->host[cb::kFalse] == 0 && n_units > 0;
   if (ctx->host[cb::kError]) {
     char msg[96];
     std::snprintf(msg, sizeof msg, "symbolic phase consistency check failed (code %lld)",
@@ -695,13 +698,11 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, const DevCSR& dB, int64_
   mark(ctx, opt, 4);
   // a pass over B's rows for the table pays once more than a few rows are cut
   // into several windows (a row's only window takes B's rows whole)
-  if (tab_pos && !(all_true && hbits) && n_units > n_heavy + n_heavy / 8) {
+  if (tab_pos && !pattern && n_units > n_heavy + n_heavy / 8) {
     tab.pos = tab_pos;
     cb::launch_split_table(dB, tab, ctx->stream, ctx->sms);
     ++launches;
   }
-  // all true: rows with stored bitmaps are read out of them, leaving no windows
-  const bool pattern = all_true && hbits && n_units > 0;
   if (pattern) {
     cb::launch_pattern_rows(dA, dB, heavy_rows, n_heavy, spans, span_counts, hbits, nnz, C->row_ptr, C->col,
                             C->val, counters, ctx->stream, ctx->sms, num_hash_max);
@@ -1251,6 +1252,7 @@ bool batched_group_graph(cb_ctx* ctx, int sr, const cb_csr& sA, const DevCSR& dB
     ensure_fused(ctx, max_rows);
     qstatus = reinterpret_cast<int*>(ctx->fsync + 4);
     CB_CUDA(cudaMemsetAsync(qstatus, 0, sizeof(int), ctx->stream));
+    CB_CUDA(cb::prepare_queue_rows(sr));
   }
   cb::prepare_dev_launchers(sr);  // kernel attributes are set outside the capture
   CB_CUDA(cudaStreamSynchronize(ctx->stream));

@@ -26,48 +26,104 @@ __global__ void k_validate(DevCSR M, int64_t nnz, int code_base, int64_t* counte
   }
 }
 
-// K1: one warp per row of A.  flops_i = sum of B row lengths over the row's
-// stored entries (the flops count of Table 1), maxb_i = the longest of them.
+// K1: flops_i = sum of B row lengths over the row's stored entries (the flops
+// count of Table 1), maxb_i = the longest of them.  One warp per row, four
+// entries per lane in flight (each costs a column and, dependent on it, its B
+// row's two pointers); rows of more than kLongRow entries are left to the end,
+// when the CTA's warps share each of them.  (A hub row of R-MAT s19, 34000
+// entries, kept one warp busy for most of the kernel's 398 us.)
+constexpr int kLongRow = 1024;
+constexpr int kLongRows = 64;  // a CTA's list; rows beyond it stay with their warp
+
+__device__ __forceinline__ void row_flops(const DevCSR& A, const DevCSR& B, int64_t p0, int64_t a1, int step,
+                                          long long& f, int& mx) {
+  for (int64_t p = p0; p < a1; p += 4 * (int64_t)step) {
+    int k[4];
+    int64_t b0[4], b1[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) k[u] = p + u * step < a1 ? A.col[p + u * step] : -1;
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      b0[u] = k[u] >= 0 ? B.rp[k[u]] : 0;
+      b1[u] = k[u] >= 0 ? row_end(B, k[u]) : 0;
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const int64_t len = b1[u] - b0[u];
+      f += len;
+      mx = max(mx, (int)min(len, (int64_t)INT_MAX));
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    f += __shfl_down_sync(0xffffffffu, f, o);
+    mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
+  }
+}
+
 __global__ void __launch_bounds__(256) k_classify_sym(DevCSR A, DevCSR B, int64_t* flops,
                                                       int32_t* maxb, int64_t* counters,
                                                       const uint8_t* skip, int64_t sym_hash_max) {
   __shared__ unsigned long long hist[kSymTiers];
   __shared__ unsigned long long total;
   __shared__ long long max_f, max_a;
+  __shared__ long long wf[8];
+  __shared__ int wm[8], longs[kLongRows], n_long;
   if (threadIdx.x < kSymTiers) hist[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     total = 0;
     max_f = 0;
     max_a = 0;
+    n_long = 0;
   }
   __syncthreads();
-  const int lane = threadIdx.x & 31;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
-  for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); i < A.nrows;
-       i += nwarps) {
+  const auto record = [&](int64_t i, int64_t entries, long long f, int mx) {
+    flops[i] = f;
+    if (maxb) maxb[i] = mx;
+    atomicAdd(&hist[skip && skip[i] ? 0 : sym_tier(min((int64_t)f, row_width(A, B, i)), sym_hash_max)], 1ull);
+    atomicAdd(&total, (unsigned long long)f);
+    atomicMax(&max_f, f);
+    atomicMax(&max_a, (long long)entries);
+  };
+  for (int64_t i = (int64_t)blockIdx.x * (blockDim.x >> 5) + warp; i < A.nrows; i += nwarps) {
     const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
+    if (a1 - a0 > kLongRow) {
+      int at = 0;
+      if (lane == 0) at = atomicAdd(&n_long, 1);
+      at = __shfl_sync(0xffffffffu, at, 0);
+      if (at < kLongRows) {
+        if (lane == 0) longs[at] = (int)i;
+        continue;
+      }
+    }
     long long f = 0;
     int mx = 0;
-    for (int64_t p = a0 + lane; p < a1; p += 32) {
-      const int k = A.col[p];
-      const int64_t len = row_end(B, k) - B.rp[k];
-      f += len;
-      mx = max(mx, (int)min(len, (int64_t)INT_MAX));
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      f += __shfl_down_sync(0xffffffffu, f, o);
-      mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
-    }
+    row_flops(A, B, a0 + lane, a1, 32, f, mx);
+    if (lane == 0) record(i, a1 - a0, f, mx);
+  }
+  __syncthreads();
+  for (int r = 0; r < min(n_long, kLongRows); ++r) {
+    const int64_t i = longs[r], a0 = A.rp[i], a1 = A.rp[i + 1];
+    long long f = 0;
+    int mx = 0;
+    row_flops(A, B, a0 + threadIdx.x, a1, 256, f, mx);
     if (lane == 0) {
-      flops[i] = f;
-      if (maxb) maxb[i] = mx;
-      atomicAdd(&hist[skip && skip[i] ? 0 : sym_tier(min((int64_t)f, row_width(A, B, i)), sym_hash_max)],
-                1ull);
-      atomicAdd(&total, (unsigned long long)f);
-      atomicMax(&max_f, f);
-      atomicMax(&max_a, (long long)(a1 - a0));
+      wf[warp] = f;
+      wm[warp] = mx;
     }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      f = 0;
+      mx = 0;
+      for (int w = 0; w < 8; ++w) {
+        f += wf[w];
+        mx = max(mx, wm[w]);
+      }
+      record(i, a1 - a0, f, mx);
+    }
+    __syncthreads();
   }
   __syncthreads();
   if (threadIdx.x < kSymTiers && hist[threadIdx.x])

@@ -32,7 +32,7 @@ def shifted(cb, M, by):
 
 
 @pytest.mark.parametrize("false_at", [None, ("A", 0), ("A", -1), ("B", 0), ("B", -1)])
-@pytest.mark.parametrize("ncols", [900, 600000])
+@pytest.mark.parametrize("ncols", [5000, 600000])
 def test_true_and_false_values(cb, ncols, false_at):
     A, B = _tiered_inputs(SR, seed=910, ncols=ncols)
     A = A.with_values(np.full(A.nnz, 1, np.uint8))
