@@ -415,7 +415,6 @@ int queue_pass(cb_ctx* ctx, int sr, const DevCSR& dA, const DevCSR& dB, int64_t 
   ensure_fused(ctx, m);
   int* st = reinterpret_cast<int*>(ctx->fsync + 4);
   CB_CUDA(cudaMemsetAsync(st, 0, sizeof(int), ctx->stream));
-  CB_CUDA(cb::prepare_queue_rows(sr));
   mark(ctx, opt, 4);
   const cudaError_t e = cb::launch_queue_rows(sr, dA, dB, m, C->row_ptr, C->col, C->val, cap,
                                               ctx->fstat, ctx->fstat_cap, ctx->fsync, st, ctx->stream,
@@ -1252,7 +1251,6 @@ bool batched_group_graph(cb_ctx* ctx, int sr, const cb_csr& sA, const DevCSR& dB
     ensure_fused(ctx, max_rows);
     qstatus = reinterpret_cast<int*>(ctx->fsync + 4);
     CB_CUDA(cudaMemsetAsync(qstatus, 0, sizeof(int), ctx->stream));
-    CB_CUDA(cb::prepare_queue_rows(sr));
   }
   cb::prepare_dev_launchers(sr);  // kernel attributes are set outside the capture
   CB_CUDA(cudaStreamSynchronize(ctx->stream));
