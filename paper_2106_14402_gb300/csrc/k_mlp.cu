@@ -36,22 +36,23 @@ constexpr int oW1 = 0, ob1 = oW1 + H * 3, oW2 = ob1 + H, ob2 = oW2 + H * H, ow3 
 static_assert(kNP == CB_MLP_NPARAM, "parameter layout");
 
 constexpr int kFwdThreads = 256;
-constexpr int kBwdThreads = 128;
-constexpr int kPad = H + 1;  // padded row stride of per-row activation tiles
+constexpr int kBatchUnit = 128;  // training batches are rounded up to a multiple of this
 
 __device__ __forceinline__ float bf16r(float v) { return __bfloat162float(__float2bfloat16_rn(v)); }
 
-// Weights staged in shared memory as floats holding bf16 values.
-struct SmemWeights {
-  float W1[H * 3], b1[H], W2[H * H], b2[H], w3[H], b3, mu[3], sg[3];
+constexpr int kNF = CB_MLP_NFEAT;  // floats per feature row
+
+// The small weights, staged in shared memory (bf16 values held as floats).
+struct SmallWeights {
+  float4 w1b[H];  // W1 row j and b1[j]
+  float b2[H], w3[H], b3, mu[3], sg[3];
 };
 
-__device__ __forceinline__ void stage_weights(SmemWeights& w, const __nv_bfloat16* wb,
-                                              const float* master, const float* norm) {
-  for (int t = threadIdx.x; t < H * 3; t += blockDim.x) w.W1[t] = __bfloat162float(wb[oW1 + t]);
-  for (int t = threadIdx.x; t < H * H; t += blockDim.x) w.W2[t] = __bfloat162float(wb[oW2 + t]);
+__device__ __forceinline__ void stage_small(SmallWeights& w, const __nv_bfloat16* wb, const float* master,
+                                            const float* norm) {
   for (int t = threadIdx.x; t < H; t += blockDim.x) {
-    w.b1[t] = master[ob1 + t];
+    w.w1b[t] = make_float4(__bfloat162float(wb[oW1 + 3 * t]), __bfloat162float(wb[oW1 + 3 * t + 1]),
+                           __bfloat162float(wb[oW1 + 3 * t + 2]), master[ob1 + t]);
     w.b2[t] = master[ob2 + t];
     w.w3[t] = __bfloat162float(wb[ow3 + t]);
   }
@@ -62,36 +63,21 @@ __device__ __forceinline__ void stage_weights(SmemWeights& w, const __nv_bfloat1
   }
 }
 
-constexpr int kNF = CB_MLP_NFEAT;  // floats per feature row
-
-__device__ __forceinline__ void features(const SmemWeights& w, const float* f, float x[3]) {
+__device__ __forceinline__ void features(const SmallWeights& w, const float* f, float x[3]) {
   const float lw = log2f(fmaxf(f[3], 1.0f));
   float l[3] = {log2f(1.0f + f[0]), log2f(1.0f + f[1]) - lw, log2f(1.0f + f[2]) - lw};
 #pragma unroll
   for (int d = 0; d < 3; ++d) x[d] = bf16r((l[d] - w.mu[d]) / w.sg[d]);
 }
 
-// Forward pass of one row; h1/h2 receive the bf16-rounded activations.
-__device__ __forceinline__ float forward_row(const SmemWeights& w, const float x[3], float* h1,
-                                             float* h2) {
-#pragma unroll 4
-  for (int j = 0; j < H; ++j) {
-    float a = w.b1[j];
-    a = fmaf(w.W1[j * 3 + 0], x[0], a);
-    a = fmaf(w.W1[j * 3 + 1], x[1], a);
-    a = fmaf(w.W1[j * 3 + 2], x[2], a);
-    h1[j] = bf16r(fmaxf(a, 0.0f));
-  }
-  float z = w.b3;
-  for (int j = 0; j < H; ++j) {
-    float a = w.b2[j];
-#pragma unroll 8
-    for (int k = 0; k < H; ++k) a = fmaf(w.W2[j * H + k], h1[k], a);
-    const float v = bf16r(fmaxf(a, 0.0f));
-    h2[j] = v;
-    z = fmaf(w.w3[j], v, z);
-  }
-  return z;
+// h1[j] of one row.
+__device__ __forceinline__ float hidden1(const SmallWeights& w, int j, const float x[3]) {
+  const float4 v = w.w1b[j];
+  float a = v.w;
+  a = fmaf(v.x, x[0], a);
+  a = fmaf(v.y, x[1], a);
+  a = fmaf(v.z, x[2], a);
+  return bf16r(fmaxf(a, 0.0f));
 }
 
 __device__ __forceinline__ int64_t size_from_logit(float z, int64_t flops, int64_t maxb,
@@ -106,134 +92,282 @@ __device__ __forceinline__ int64_t size_from_logit(float z, int64_t flops, int64
   return est;
 }
 
-// K8: one thread per row.
-__global__ void __launch_bounds__(kFwdThreads) k_mlp_predict(const __nv_bfloat16* wb,
-                                                             const float* master, const float* norm,
-                                                             const float* feat, int64_t m,
-                                                             int64_t ncols, float* z_out,
-                                                             int64_t* pred_out) {
-  __shared__ SmemWeights w;
-  __shared__ float h1s[kFwdThreads * kPad];
-  stage_weights(w, wb, master, norm);
+// K8: a warp per 32 rows.  Every sum runs over its inputs in ascending order
+// in fp32 (one rounding per product), whichever thread holds it, so logits do
+// not depend on the layout.  The 64 x 64 layer is an outer-product loop on
+// 8 rows x 8 outputs per lane: h1 lies [input][row] in shared memory, W2
+// transposed, and each step of 64 FMAs per lane reads four 16-byte vectors
+// (shared-memory bandwidth and FMA issue are about even; one thread per row,
+// which read two shared words per FMA, took 379 us for 524288 rows).
+constexpr int kFwdWarps = kFwdThreads / 32;
+constexpr int kRowPad = H + 4;  // row stride of h2: 16-byte reads of 8 rows meet all banks
+struct PredictSmem {
+  SmallWeights s;
+  float w2t[H * H];                    // [input][output]
+  float h[kFwdWarps][32 * kRowPad];    // a warp's h1 [input][32 rows], then h2 [row][kRowPad]
+};
+
+__global__ void __launch_bounds__(kFwdThreads, 2) k_mlp_predict(const __nv_bfloat16* wb, const float* master,
+                                                                const float* norm, const float* feat,
+                                                                int64_t m, int64_t ncols, float* z_out,
+                                                                int64_t* pred_out) {
+  extern __shared__ __align__(16) unsigned char mlp_smem[];
+  PredictSmem& w = *reinterpret_cast<PredictSmem*>(mlp_smem);
+  stage_small(w.s, wb, master, norm);
+  for (int t = threadIdx.x; t < H * H; t += kFwdThreads)
+    w.w2t[(t % H) * H + t / H] = __bfloat162float(wb[oW2 + t]);
   __syncthreads();
-  float h2[H];
-  float* h1 = h1s + threadIdx.x * kPad;
-  for (int64_t r = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; r < m;
-       r += (int64_t)gridDim.x * blockDim.x) {
-    float x[3];
-    const float* f = feat + kNF * r;
-    features(w, f, x);
-    const float z = forward_row(w, x, h1, h2);
-    if (z_out) z_out[r] = z;
-    if (pred_out) pred_out[r] = size_from_logit(z, (int64_t)f[1], (int64_t)f[2], (int64_t)f[3], ncols);
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int rg = lane >> 3, jg = lane & 7;  // rows 8 rg .. + 7, outputs 4 jg .. + 3 and 32 + 4 jg .. + 3
+  float* const h = w.h[warp];
+  for (int64_t r0 = ((int64_t)blockIdx.x * kFwdWarps + warp) * 32; r0 < m;
+       r0 += (int64_t)gridDim.x * kFwdThreads) {
+    const int64_t r = r0 + lane;
+    float f[kNF] = {0.0f, 0.0f, 0.0f, 1.0f}, x[3];
+    if (r < m) {
+#pragma unroll
+      for (int d = 0; d < kNF; ++d) f[d] = feat[kNF * r + d];
+    }
+    features(w.s, f, x);
+#pragma unroll 4
+    for (int j = 0; j < H; ++j) h[32 * j + lane] = hidden1(w.s, j, x);
+    __syncwarp();
+    float acc[8][8];  // [row][output]
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      const float b = w.s.b2[(q < 4 ? 0 : 28) + 4 * jg + q];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc[i][q] = b;
+    }
+#pragma unroll 2
+    for (int k = 0; k < H; ++k) {
+      float a[8], b[8];
+      *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(h + 32 * k + 8 * rg);
+      *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(h + 32 * k + 8 * rg + 4);
+      *reinterpret_cast<float4*>(b) = *reinterpret_cast<const float4*>(w.w2t + H * k + 4 * jg);
+      *reinterpret_cast<float4*>(b + 4) = *reinterpret_cast<const float4*>(w.w2t + H * k + 32 + 4 * jg);
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+#pragma unroll
+        for (int q = 0; q < 8; ++q) acc[i][q] = fmaf(b[q], a[i], acc[i][q]);
+    }
+    __syncwarp();  // h1 is read; h2 takes its place
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q) acc[i][q] = bf16r(fmaxf(acc[i][q], 0.0f));
+      float* const o = h + (8 * rg + i) * kRowPad + 4 * jg;
+      *reinterpret_cast<float4*>(o) = make_float4(acc[i][0], acc[i][1], acc[i][2], acc[i][3]);
+      *reinterpret_cast<float4*>(o + 32) = make_float4(acc[i][4], acc[i][5], acc[i][6], acc[i][7]);
+    }
+    __syncwarp();
+    float z = w.s.b3;
+#pragma unroll
+    for (int j = 0; j < H; j += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(h + lane * kRowPad + j);
+      z = fmaf(w.s.w3[j], v.x, z);
+      z = fmaf(w.s.w3[j + 1], v.y, z);
+      z = fmaf(w.s.w3[j + 2], v.z, z);
+      z = fmaf(w.s.w3[j + 3], v.w, z);
+    }
+    if (r < m) {
+      if (z_out) z_out[r] = z;
+      if (pred_out) pred_out[r] = size_from_logit(z, (int64_t)f[1], (int64_t)f[2], (int64_t)f[3], ncols);
+    }
+    __syncwarp();  // h2 is read; the next rows' h1 takes its place
   }
 }
 
 // K9: forward + pinball loss + backward for rows [r0, r0 + n).  Gradient sums
 // (not yet divided by the number of live rows) are added to grad[0..kNP),
 // the loss sum to stat[0] and the live-row count to stat[1].
-__global__ void __launch_bounds__(kBwdThreads) k_mlp_grad(const __nv_bfloat16* wb,
-                                                          const float* master, const float* norm,
-                                                          const float* feat, const int64_t* nnz,
-                                                          int64_t r0, int64_t n, float tau,
+// A CTA takes 64 rows at a time: both 64 x 64 x 64 products of the layer (and
+// the third, its weight gradient) run on 4 x 4 outputs per thread from
+// shared-memory tiles [unit][row], and the weight gradient stays in registers
+// until the CTA's last rows.  8192 rows, a training mini-batch, then run on
+// 128 SMs at once.  (128 rows per 128-thread CTA, a row per thread with its
+// layer loops serial, kept 64 SMs busy for 94 us.)
+constexpr int kBwdRows = 64, kBwdThreads = 256;
+constexpr int kTile = kBwdRows + 4;  // row stride of the tiles
+struct GradSmem {
+  SmallWeights s;
+  float w2[H * H], w2t[H * H];   // [output][input], [input][output]
+  float h1[H * kTile], d2[H * kTile], d1[H * kTile];  // [unit][row]; d2 holds h2 first
+  float x[3][kBwdRows], dz[kBwdRows];
+};
+
+__global__ void __launch_bounds__(kBwdThreads) k_mlp_grad(const __nv_bfloat16* wb, const float* master,
+                                                          const float* norm, const float* feat,
+                                                          const int64_t* nnz, int64_t r0, int64_t n, float tau,
                                                           float* grad, double* stat) {
-  constexpr int T = kBwdThreads;
-  __shared__ SmemWeights w;
-  extern __shared__ float tiles[];  // h1, h2, dh2, dh1: [T][kPad] each; x: [T][3]; dz: [T]
-  float* h1 = tiles;
-  float* h2 = h1 + T * kPad;
-  float* dh2 = h2 + T * kPad;
-  float* dh1 = dh2 + T * kPad;
-  float* xs = dh1 + T * kPad;
-  float* dzs = xs + T * 3;
-  __shared__ float loss_part[T];
-  __shared__ int live_part[T];
-  stage_weights(w, wb, master, norm);
-  __syncthreads();
-  const int t = threadIdx.x;
-  const int64_t base = r0 + (int64_t)blockIdx.x * T;
-  const int64_t r = base + t;
-  float dz = 0.0f, loss = 0.0f;
-  int live = 0;
-  float* my1 = h1 + t * kPad;
-  float* my2 = h2 + t * kPad;
-  if (r < r0 + n) {
-    float x[3];
-    features(w, feat + kNF * r, x);
-    xs[t * 3 + 0] = x[0];
-    xs[t * 3 + 1] = x[1];
-    xs[t * 3 + 2] = x[2];
-    const float z = forward_row(w, x, my1, my2);
-    const float fl = feat[kNF * r + 1];
-    if (fl > 0.0f) {
-      live = 1;
-      const float ls = -(fmaxf(-z, 0.0f) + log1pf(expf(-fabsf(z))));  // log sigmoid(z)
-      const float e = log2f((float)nnz[r] / fl) - ls * 1.4426950408889634f;
-      loss = e >= 0.0f ? tau * e : (tau - 1.0f) * e;
-      const float sig = 1.0f / (1.0f + expf(-z));
-      dz = (e >= 0.0f ? tau : tau - 1.0f) * (-(1.0f - sig) * 1.4426950408889634f);
-    }
-  } else {
-    for (int j = 0; j < H; ++j) my1[j] = my2[j] = 0.0f;
-    xs[t * 3 + 0] = xs[t * 3 + 1] = xs[t * 3 + 2] = 0.0f;
+  extern __shared__ __align__(16) unsigned char mlp_smem[];
+  GradSmem& w = *reinterpret_cast<GradSmem*>(mlp_smem);
+  stage_small(w.s, wb, master, norm);
+  for (int t = threadIdx.x; t < H * H; t += kBwdThreads) {
+    const float v = __bfloat162float(wb[oW2 + t]);
+    w.w2[t] = v;
+    w.w2t[(t % H) * H + t / H] = v;
   }
-  dzs[t] = dz;
-  loss_part[t] = loss;
-  live_part[t] = live;
-  float* myd2 = dh2 + t * kPad;
-  for (int j = 0; j < H; ++j) myd2[j] = my2[j] > 0.0f ? dz * w.w3[j] : 0.0f;
-  float* myd1 = dh1 + t * kPad;
-  for (int k = 0; k < H; ++k) {
-    float a = 0.0f;
+  const int tid = threadIdx.x;
+  const int lo4 = 4 * (tid & 15), hi4 = 4 * (tid >> 4);  // 4 x 4 tile: rows (or inputs), units
+  const int unit = tid >> 2, part = tid & 3;             // sums over 16 rows of one unit
+  float gw2[4][4] = {};                                  // [output hi4 + a][input tid % 16 + 16 b]
+  float gw3 = 0.0f, gb2 = 0.0f, gb1 = 0.0f, gw1[3] = {0.0f, 0.0f, 0.0f}, gb3 = 0.0f;
+  double loss_sum = 0.0;
+  int live_sum = 0;
+  for (int64_t base = (int64_t)blockIdx.x * kBwdRows; base < n; base += (int64_t)gridDim.x * kBwdRows) {
+    __syncthreads();  // weights staged; the last tile's readers are done
+    {
+      const int row = tid & (kBwdRows - 1), j0 = (tid / kBwdRows) * 16;
+      const int64_t r = base + row;
+      float x[3] = {0.0f, 0.0f, 0.0f};
+      if (r < n) features(w.s, feat + kNF * (r0 + r), x);
+#pragma unroll 4
+      for (int j = j0; j < j0 + 16; ++j) w.h1[j * kTile + row] = r < n ? hidden1(w.s, j, x) : 0.0f;
+      if (tid < kBwdRows) {
+        w.x[0][row] = x[0];
+        w.x[1][row] = x[1];
+        w.x[2][row] = x[2];
+      }
+    }
+    __syncthreads();
+    {  // h2[hi4 + b][lo4 + a]
+      float acc[4][4];
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int a = 0; a < 4; ++a) acc[b][a] = w.s.b2[hi4 + b];
+#pragma unroll 4
+      for (int k = 0; k < H; ++k) {
+        float h[4], v[4];
+        *reinterpret_cast<float4*>(h) = *reinterpret_cast<const float4*>(w.h1 + k * kTile + lo4);
+        *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(w.w2t + k * H + hi4);
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int a = 0; a < 4; ++a) acc[b][a] = fmaf(v[b], h[a], acc[b][a]);
+      }
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+        *reinterpret_cast<float4*>(w.d2 + (hi4 + b) * kTile + lo4) =
+            make_float4(bf16r(fmaxf(acc[b][0], 0.0f)), bf16r(fmaxf(acc[b][1], 0.0f)),
+                        bf16r(fmaxf(acc[b][2], 0.0f)), bf16r(fmaxf(acc[b][3], 0.0f)));
+    }
+    __syncthreads();
+    if (tid < kBwdRows) {  // the logit, its loss and slope
+      float z = w.s.b3;
 #pragma unroll 8
-    for (int j = 0; j < H; ++j) a = fmaf(myd2[j], w.W2[j * H + k], a);
-    myd1[k] = my1[k] > 0.0f ? a : 0.0f;
-  }
-  __syncthreads();
-  // weight-gradient reductions over the block's rows
-  {
-    // W2: thread pair (j, half) sums 32 entries over T rows
-    const int j = t >> 1, k0 = (t & 1) * (H / 2);
-    float acc[H / 2];
-#pragma unroll
-    for (int q = 0; q < H / 2; ++q) acc[q] = 0.0f;
-    for (int rr = 0; rr < T; ++rr) {
-      const float d = dh2[rr * kPad + j];
-#pragma unroll
-      for (int q = 0; q < H / 2; ++q) acc[q] = fmaf(d, h1[rr * kPad + k0 + q], acc[q]);
+      for (int j = 0; j < H; ++j) z = fmaf(w.s.w3[j], w.d2[j * kTile + tid], z);
+      float dz = 0.0f;
+      const int64_t r = base + tid;
+      if (r < n) {
+        const float fl = feat[kNF * (r0 + r) + 1];
+        if (fl > 0.0f) {
+          const float ls = -(fmaxf(-z, 0.0f) + log1pf(expf(-fabsf(z))));  // log sigmoid(z)
+          const float e = log2f((float)nnz[r0 + r] / fl) - ls * 1.4426950408889634f;
+          loss_sum += (double)(e >= 0.0f ? tau * e : (tau - 1.0f) * e);
+          ++live_sum;
+          const float sig = 1.0f / (1.0f + expf(-z));
+          dz = (e >= 0.0f ? tau : tau - 1.0f) * (-(1.0f - sig) * 1.4426950408889634f);
+        }
+      }
+      w.dz[tid] = dz;
+      gb3 += dz;
     }
+    __syncthreads();
+    {  // h2 -> its gradient in place, with the sums that need it
+      const float w3 = w.s.w3[unit];
+#pragma unroll 4
+      for (int t = 0; t < 16; ++t) {
+        const int row = 16 * part + t;
+        float* const p = w.d2 + unit * kTile + row;
+        const float h = *p, dz = w.dz[row];
+        gw3 = fmaf(dz, h, gw3);
+        const float d = h > 0.0f ? dz * w3 : 0.0f;
+        gb2 += d;
+        *p = d;
+      }
+    }
+    __syncthreads();
+    {  // d1[hi4 + b][lo4 + a], and the weight gradient's outer products
+      float acc[4][4] = {};
+#pragma unroll 4
+      for (int j = 0; j < H; ++j) {
+        float d[4], v[4];
+        *reinterpret_cast<float4*>(d) = *reinterpret_cast<const float4*>(w.d2 + j * kTile + lo4);
+        *reinterpret_cast<float4*>(v) = *reinterpret_cast<const float4*>(w.w2 + j * H + hi4);
 #pragma unroll
-    for (int q = 0; q < H / 2; ++q) atomicAdd(&grad[oW2 + j * H + k0 + q], acc[q]);
-  }
-  if (t < H) {
-    float gw3 = 0.0f, gb2 = 0.0f, gb1 = 0.0f, g1[3] = {0.0f, 0.0f, 0.0f};
-    for (int rr = 0; rr < T; ++rr) {
-      gw3 = fmaf(dzs[rr], h2[rr * kPad + t], gw3);
-      gb2 += dh2[rr * kPad + t];
-      const float d1 = dh1[rr * kPad + t];
-      gb1 += d1;
-      g1[0] = fmaf(d1, xs[rr * 3 + 0], g1[0]);
-      g1[1] = fmaf(d1, xs[rr * 3 + 1], g1[1]);
-      g1[2] = fmaf(d1, xs[rr * 3 + 2], g1[2]);
+        for (int b = 0; b < 4; ++b)
+#pragma unroll
+          for (int a = 0; a < 4; ++a) acc[b][a] = fmaf(d[a], v[b], acc[b][a]);
+      }
+#pragma unroll
+      for (int b = 0; b < 4; ++b) {
+        const float4 h = *reinterpret_cast<const float4*>(w.h1 + (hi4 + b) * kTile + lo4);
+        *reinterpret_cast<float4*>(w.d1 + (hi4 + b) * kTile + lo4) =
+            make_float4(h.x > 0.0f ? acc[b][0] : 0.0f, h.y > 0.0f ? acc[b][1] : 0.0f,
+                        h.z > 0.0f ? acc[b][2] : 0.0f, h.w > 0.0f ? acc[b][3] : 0.0f);
+      }
+#pragma unroll 2
+      for (int r = 0; r < kBwdRows; r += 4) {
+        float4 d[4], h[4];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) d[a] = *reinterpret_cast<const float4*>(w.d2 + (hi4 + a) * kTile + r);
+#pragma unroll
+        for (int b = 0; b < 4; ++b)
+          h[b] = *reinterpret_cast<const float4*>(w.h1 + ((tid & 15) + 16 * b) * kTile + r);
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int b = 0; b < 4; ++b) {
+            gw2[a][b] = fmaf(d[a].x, h[b].x, gw2[a][b]);
+            gw2[a][b] = fmaf(d[a].y, h[b].y, gw2[a][b]);
+            gw2[a][b] = fmaf(d[a].z, h[b].z, gw2[a][b]);
+            gw2[a][b] = fmaf(d[a].w, h[b].w, gw2[a][b]);
+          }
+      }
     }
-    atomicAdd(&grad[ow3 + t], gw3);
-    atomicAdd(&grad[ob2 + t], gb2);
-    atomicAdd(&grad[ob1 + t], gb1);
-    atomicAdd(&grad[oW1 + t * 3 + 0], g1[0]);
-    atomicAdd(&grad[oW1 + t * 3 + 1], g1[1]);
-    atomicAdd(&grad[oW1 + t * 3 + 2], g1[2]);
-  }
-  if (t == H) {
-    float gb3 = 0.0f, ls = 0.0f;
-    int lv = 0;
-    for (int rr = 0; rr < T; ++rr) {
-      gb3 += dzs[rr];
-      ls += loss_part[rr];
-      lv += live_part[rr];
+    __syncthreads();
+#pragma unroll 4
+    for (int t = 0; t < 16; ++t) {
+      const int row = 16 * part + t;
+      const float d = w.d1[unit * kTile + row];
+      gb1 += d;
+      gw1[0] = fmaf(d, w.x[0][row], gw1[0]);
+      gw1[1] = fmaf(d, w.x[1][row], gw1[1]);
+      gw1[2] = fmaf(d, w.x[2][row], gw1[2]);
     }
-    atomicAdd(&grad[ob3], gb3);
-    atomicAdd(&stat[0], (double)ls);
-    atomicAdd(&stat[1], (double)lv);
+  }
+#pragma unroll
+  for (int a = 0; a < 4; ++a)
+#pragma unroll
+    for (int b = 0; b < 4; ++b) atomicAdd(&grad[oW2 + (hi4 + a) * H + (tid & 15) + 16 * b], gw2[a][b]);
+  float sums[6] = {gw3, gb2, gb1, gw1[0], gw1[1], gw1[2]};
+#pragma unroll
+  for (int q = 0; q < 6; ++q) {
+    sums[q] += __shfl_xor_sync(0xffffffffu, sums[q], 1);
+    sums[q] += __shfl_xor_sync(0xffffffffu, sums[q], 2);
+  }
+  if (part == 0) {
+    atomicAdd(&grad[ow3 + unit], sums[0]);
+    atomicAdd(&grad[ob2 + unit], sums[1]);
+    atomicAdd(&grad[ob1 + unit], sums[2]);
+    atomicAdd(&grad[oW1 + unit * 3 + 0], sums[3]);
+    atomicAdd(&grad[oW1 + unit * 3 + 1], sums[4]);
+    atomicAdd(&grad[oW1 + unit * 3 + 2], sums[5]);
+  }
+  if (tid < kBwdRows) {
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+      gb3 += __shfl_down_sync(0xffffffffu, gb3, d);
+      loss_sum += __shfl_down_sync(0xffffffffu, loss_sum, d);
+      live_sum += __shfl_down_sync(0xffffffffu, live_sum, d);
+    }
+    if ((tid & 31) == 0) {
+      atomicAdd(&grad[ob3], gb3);
+      atomicAdd(&stat[0], loss_sum);
+      atomicAdd(&stat[1], (double)live_sum);
+    }
   }
 }
 
@@ -293,7 +427,15 @@ __global__ void k_row_features(DevCSR A, const int64_t* flops, const int32_t* ma
   }
 }
 
-constexpr size_t kGradSmem = (size_t)kBwdThreads * (4 * kPad + 4) * sizeof(float);
+// Launch over n rows; the shared-memory limit is the current device's.
+void run_grad(const __nv_bfloat16* wb, const float* master, const float* norm, const float* feat,
+              const int64_t* nnz, int64_t r0, int64_t n, float tau, float* grad, double* stat, int sms,
+              cudaStream_t s) {
+  cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(GradSmem));
+  const int64_t tiles = (n + kBwdRows - 1) / kBwdRows, most = 2 * (int64_t)sms;
+  k_mlp_grad<<<(unsigned)(tiles < most ? tiles : most), kBwdThreads, sizeof(GradSmem), s>>>(
+      wb, master, norm, feat, nnz, r0, n, tau, grad, stat);
+}
 
 }  // namespace
 
@@ -307,8 +449,9 @@ void launch_row_features(const DevCSR& A, const int64_t* flops, const int32_t* m
 void launch_mlp_predict(const void* wb, const float* master, const float* norm, const float* feat,
                         int64_t m, int64_t ncols, float* z, int64_t* pred, cudaStream_t s, int sms) {
   if (m == 0) return;
-  int64_t g = (m + kFwdThreads - 1) / kFwdThreads;
-  k_mlp_predict<<<(int)(g < sms * 4 ? g : sms * 4), kFwdThreads, 0, s>>>(
+  cudaFuncSetAttribute(k_mlp_predict, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(PredictSmem));
+  const int64_t g = (m + kFwdThreads - 1) / kFwdThreads;
+  k_mlp_predict<<<(int)(g < sms * 2 ? g : sms * 2), kFwdThreads, sizeof(PredictSmem), s>>>(
       static_cast<const __nv_bfloat16*>(wb), master, norm, feat, m, ncols, z, pred);
 }
 
@@ -439,19 +582,11 @@ extern "C" int cb_mlp_grad(cb_ctx* ctx, const cb_mlp* m, const float* feat, cons
   using namespace cb;
   if (!ctx || !m || nrows < 0 || (nrows > 0 && (!feat || !nnz)) || !grad) return CB_ERR_ARG;
   cudaStream_t s = ctx_stream(ctx);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem);
-    attr = true;
-  }
   if (cudaMemsetAsync(m->grad, 0, kNP * sizeof(float), s) != cudaSuccess ||
       cudaMemsetAsync(m->stat, 0, 2 * sizeof(double), s) != cudaSuccess)
     return CB_ERR_CUDA;
-  if (nrows > 0) {
-    const int64_t blocks = (nrows + kBwdThreads - 1) / kBwdThreads;
-    k_mlp_grad<<<(unsigned)blocks, kBwdThreads, kGradSmem, s>>>(m->wb, m->master, m->norm, feat, nnz,
-                                                                 0, nrows, tau, m->grad, m->stat);
-  }
+  if (nrows > 0)
+    run_grad(m->wb, m->master, m->norm, feat, nnz, 0, nrows, tau, m->grad, m->stat, ctx_sms(ctx), s);
   k_mlp_scale<<<8, 256, 0, s>>>(m->grad, m->stat, grad, loss);
   const bool ok = cudaGetLastError() == cudaSuccess &&
                   cudaMemsetAsync(m->grad, 0, kNP * sizeof(float), s) == cudaSuccess &&
@@ -466,28 +601,21 @@ extern "C" int cb_mlp_train(cb_ctx* ctx, cb_mlp* m, const float* feat, const int
   if (!ctx || !m || nrows <= 0 || !feat || !nnz || epochs < 0 || batch <= 0 || !(lr > 0.0f))
     return CB_ERR_ARG;
   cudaStream_t s = ctx_stream(ctx);
-  static bool attr = false;
-  if (!attr) {
-    cudaFuncSetAttribute(k_mlp_grad, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kGradSmem);
-    attr = true;
-  }
-  if (batch % kBwdThreads) batch += kBwdThreads - batch % kBwdThreads;
+  if (batch % kBatchUnit) batch += kBatchUnit - batch % kBatchUnit;
   if (cudaMemsetAsync(m->grad, 0, kNP * sizeof(float), s) != cudaSuccess ||
       cudaMemsetAsync(m->stat, 0, 4 * sizeof(double), s) != cudaSuccess)
     return CB_ERR_CUDA;
   for (int ep = 0; ep < epochs; ++ep) {
     // each epoch starts the batch sequence at a different offset
-    const int64_t shift = ((int64_t)ep * 7919 * kBwdThreads) % nrows;
+    const int64_t shift = ((int64_t)ep * 7919 * kBatchUnit) % nrows;
     for (int64_t done = 0; done < nrows; done += batch) {
       const int64_t start = (shift + done) % nrows;
       int64_t n = batch < nrows - done ? batch : nrows - done;
       // a batch that runs past the end wraps to the front in two launches
       const int64_t n1 = n < nrows - start ? n : nrows - start;
-      k_mlp_grad<<<(unsigned)((n1 + kBwdThreads - 1) / kBwdThreads), kBwdThreads, kGradSmem, s>>>(
-          m->wb, m->master, m->norm, feat, nnz, start, n1, tau, m->grad, m->stat);
+      run_grad(m->wb, m->master, m->norm, feat, nnz, start, n1, tau, m->grad, m->stat, ctx_sms(ctx), s);
       if (n > n1)
-        k_mlp_grad<<<(unsigned)((n - n1 + kBwdThreads - 1) / kBwdThreads), kBwdThreads, kGradSmem,
-                     s>>>(m->wb, m->master, m->norm, feat, nnz, 0, n - n1, tau, m->grad, m->stat);
+        run_grad(m->wb, m->master, m->norm, feat, nnz, 0, n - n1, tau, m->grad, m->stat, ctx_sms(ctx), s);
       ++m->step;
       k_mlp_adam<<<1, 1024, 0, s>>>(m->master, m->wb, m->mom, m->vel, m->grad, m->stat,
                                     m->stat + 2, lr, 0.9f, 0.999f, m->step);
