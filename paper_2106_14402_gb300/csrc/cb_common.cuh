@@ -494,6 +494,11 @@ __device__ __forceinline__ int64_t row_end(const DevCSR& M, int64_t k) {
   return M.rpe ? M.rpe[k] : M.rp[k + 1];
 }
 
+// Whether a validation queued before this kernel failed (uniform).
+__device__ __forceinline__ bool gated(const int64_t* gate) {
+  return gate && *reinterpret_cast<const volatile int64_t*>(gate) != 0;
+}
+
 // Output width of row i of A.B: A.rcols[i] when set (stacked batches, where
 // each product keeps its own columns), else the width of B's view.
 __device__ __forceinline__ int64_t row_width(const DevCSR& A, const DevCSR& B, int64_t i) {

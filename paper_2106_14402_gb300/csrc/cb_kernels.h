@@ -68,6 +68,9 @@ struct DevCSR {
   // A only: per-row output width (columns of row i lie in [0, rcols[i]));
   // nullptr = the width of B's view
   const int32_t* rcols = nullptr;
+  // error word of a validation queued before the kernel (nullptr: none): the
+  // kernels that run before the host has read it do nothing when it is set
+  const int64_t* gate = nullptr;
 };
 
 // Counters block in device memory (int64 each).
@@ -91,9 +94,9 @@ enum Counter {
 };
 
 // Validation of one CSR operand: row_ptr[0] == 0, non-decreasing,
-// row_ptr[n] == nnz, 0 <= col < ncols.  Sets counters[kError] to a nonzero
-// code on failure (1 = row_ptr, 2 = column), kErrDetail to an offending index.
-void launch_validate(const DevCSR& M, int64_t nnz, int code_base, int64_t* counters,
+// row_ptr[n] == nnz, 0 <= col < ncols.  Sets err[0] to a nonzero code on
+// failure (1 = row_ptr, 2 = column, plus code_base), err[1] to an offending index.
+void launch_validate(const DevCSR& M, int64_t nnz, int code_base, int64_t* err,
                      cudaStream_t s, int sms);
 
 // K1: flops_i, maxB_i and the symbolic tier histogram; total flops.
@@ -104,7 +107,8 @@ void launch_classify_sym(const DevCSR& A, const DevCSR& B, int64_t* flops, int32
 void launch_scatter_sym(int64_t m, int64_t ncols, const int64_t* flops, int32_t* perm,
                         int64_t* nnz, int64_t* counters, cudaStream_t s, int sms,
                         const uint8_t* skip = nullptr, const int64_t* preset = nullptr,
-                        int64_t sym_hash_max = 512, const int32_t* rcols = nullptr);
+                        int64_t sym_hash_max = 512, const int32_t* rcols = nullptr,
+                        const int64_t* gate = nullptr);
 
 // K4: out[0] = 0, out[i+1] = out[i] + in[i]; partial needs scan_partials(n) int64.
 // Entries per scan tile (one partial sum per tile); the allocation-free
@@ -228,7 +232,8 @@ void launch_mlp_predict(const void* wb, const float* master, const float* norm, 
 // all zero when first used; they must not be shared by launches in flight.
 // sync: [0] launch epoch, [1] finished CTAs, [2..3] nnz(C) of the last
 // launch (int64), [6..7] its product count, [8..9] the product accumulator;
-// words 4 and 5 are free for the caller (the context keeps a status there).
+// words 4 and 5 are free for the caller (the context keeps a status there),
+// and so are 12..15 (the context's validation error).
 // SpMSpV steps (k_spmspv.cu): 0 SPA init over n, 1 chunk counts of the x
 // entries (bad indices set *err), 2 push into the SPA (cpre = scanned chunk
 // counts, cpre[nx] = total), 3 popcounts of the touched bitmap, 4 compaction

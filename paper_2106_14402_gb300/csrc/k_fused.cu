@@ -132,6 +132,7 @@ __global__ void __launch_bounds__(kFThreads, 4) k_fused(DevCSR A, DevCSR B, int6
   typedef typename S::A Acc;
   typedef typename S::TA TA;
   typedef typename S::TB TB;
+  if (gated(A.gate)) return;  // every CTA: the launch leaves no trace
   constexpr int F = G * kFE;            // products per row at most
   constexpr int LOGF = clog2(F);
   constexpr int RPW = 32 / G;           // rows per warp

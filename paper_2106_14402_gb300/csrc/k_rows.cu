@@ -9,21 +9,27 @@ namespace cb {
 
 namespace {
 
-__device__ __forceinline__ void set_error(int64_t* counters, int64_t code, int64_t detail) {
-  if (atomicCAS((unsigned long long*)&counters[kError], 0ull, (unsigned long long)code) == 0ull)
-    counters[kErrDetail] = detail;
+__device__ __forceinline__ void set_error(int64_t* err, int64_t code, int64_t detail) {
+  if (atomicCAS((unsigned long long*)&err[0], 0ull, (unsigned long long)code) == 0ull) err[1] = detail;
 }
 
-__global__ void k_validate(DevCSR M, int64_t nnz, int code_base, int64_t* counters) {
+// Columns are read four at a time when they start on a 16-byte boundary.
+__global__ void __launch_bounds__(256) k_validate(DevCSR M, int64_t nnz, int code_base, int64_t* err) {
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-  if (tid == 0 && (M.rp[0] != 0 || M.rp[M.nrows] != nnz)) set_error(counters, code_base + 1, 0);
+  if (tid == 0 && (M.rp[0] != 0 || M.rp[M.nrows] != nnz)) set_error(err, code_base + 1, 0);
   for (int64_t i = tid; i < M.nrows; i += stride)
-    if (M.rp[i + 1] < M.rp[i]) set_error(counters, code_base + 1, i);
-  for (int64_t q = tid; q < nnz; q += stride) {
-    int32_t c = M.col[q];
-    if (c < 0 || (int64_t)c >= M.ncols) set_error(counters, code_base + 2, q);
+    if (M.rp[i + 1] < M.rp[i]) set_error(err, code_base + 1, i);
+  const unsigned n = (unsigned)M.ncols;
+  const int64_t quads = (reinterpret_cast<uintptr_t>(M.col) & 15) ? 0 : nnz >> 2;
+  const uint4* v = reinterpret_cast<const uint4*>(M.col);
+  for (int64_t t = tid; t < quads; t += stride) {
+    const uint4 c = __ldg(v + t);
+    if (max(max(c.x, c.y), max(c.z, c.w)) >= n)
+      set_error(err, code_base + 2, 4 * t + (c.x >= n ? 0 : c.y >= n ? 1 : c.z >= n ? 2 : 3));
   }
+  for (int64_t q = 4 * quads + tid; q < nnz; q += stride)
+    if ((unsigned)M.col[q] >= n) set_error(err, code_base + 2, q);
 }
 
 // K1: flops_i = sum of B row lengths over the row's stored entries (the flops
@@ -69,6 +75,7 @@ __global__ void __launch_bounds__(256) k_classify_sym(DevCSR A, DevCSR B, int64_
   __shared__ long long max_f, max_a;
   __shared__ long long wf[8];
   __shared__ int wm[8], longs[kLongRows], n_long;
+  if (gated(A.gate)) return;
   if (threadIdx.x < kSymTiers) hist[threadIdx.x] = 0;
   if (threadIdx.x == 0) {
     total = 0;
@@ -141,6 +148,7 @@ struct TierBySize {
   const uint8_t* skip;         // rows with skip[i] != 0 are left out (tier 0)
   const int32_t* rcap = nullptr;  // per-row cap (replaces cap when set)
   int64_t* counters = nullptr;    // symbolic tiers: tier 4 in two classes (k_tier_scatter)
+  const int64_t* gate = nullptr;
   __device__ __forceinline__ int operator()(int64_t i) const {
     if (skip && skip[i]) return 0;
     const int64_t u = min(v[i], rcap ? (int64_t)rcap[i] : cap);
@@ -176,6 +184,7 @@ __global__ void __launch_bounds__(256) k_tier_scatter(int64_t m, TierBySize tier
                                                       int64_t* zero_nnz, const int64_t* preset) {
   __shared__ int local[6];  // tiers; 5 = the rows of tier 4 placed from its end
   __shared__ long long base[6];
+  if (gated(tier.gate)) return;
   if (threadIdx.x < 6) local[threadIdx.x] = 0;
   __syncthreads();
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -345,9 +354,9 @@ inline int grid_for(int64_t work, int per_block, int cap) {
 
 }  // namespace
 
-void launch_validate(const DevCSR& M, int64_t nnz, int code_base, int64_t* counters,
+void launch_validate(const DevCSR& M, int64_t nnz, int code_base, int64_t* err,
                      cudaStream_t s, int sms) {
-  k_validate<<<grid_for(nnz + M.nrows, 256, sms * 8), 256, 0, s>>>(M, nnz, code_base, counters);
+  k_validate<<<grid_for(nnz / 4 + M.nrows, 256, sms * 8), 256, 0, s>>>(M, nnz, code_base, err);
 }
 
 void launch_classify_sym(const DevCSR& A, const DevCSR& B, int64_t* flops, int32_t* maxb,
@@ -360,8 +369,8 @@ void launch_classify_sym(const DevCSR& A, const DevCSR& B, int64_t* flops, int32
 void launch_scatter_sym(int64_t m, int64_t ncols, const int64_t* flops, int32_t* perm,
                         int64_t* nnz, int64_t* counters, cudaStream_t s, int,
                         const uint8_t* skip, const int64_t* preset, int64_t sym_hash_max,
-                        const int32_t* rcols) {
-  TierBySize t{flops, ncols, kSymWarpMax, kSymSmallMax, sym_hash_max, skip, rcols, counters};
+                        const int32_t* rcols, const int64_t* gate) {
+  TierBySize t{flops, ncols, kSymWarpMax, kSymSmallMax, sym_hash_max, skip, rcols, counters, gate};
   k_tier_scatter<<<grid_for(m, 256, 1 << 30), 256, 0, s>>>(m, t, perm, counters + kCntSym,
                                                             counters + kCurSym, nnz, preset);
 }

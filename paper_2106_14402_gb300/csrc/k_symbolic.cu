@@ -219,6 +219,7 @@ __global__ void __launch_bounds__(256) k_check_sorted(DevCSR B, int64_t* counter
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
   int bad = 0;
+  if (gated(B.gate)) return;
   for (int64_t r = (int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); r < B.nrows;
        r += nwarps) {
     const int64_t q1 = row_end(B, r);
