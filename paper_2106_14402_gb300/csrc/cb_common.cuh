@@ -166,8 +166,8 @@ template <> struct Sem<3> {  // (min,+) over uint32, + saturating at UINT32_MAX
   static constexpr bool kUsesA = true;
   __device__ static __forceinline__ A ident() { return 0xFFFFFFFFu; }
   __device__ static __forceinline__ A mul(TA a, TB b) {
-    unsigned s = a + b;
-    return s < a ? 0xFFFFFFFFu : s;
+    const unsigned room = ~a;  // what a + b may add without saturating
+    return a + (b < room ? b : room);
   }
   __device__ static __forceinline__ A add(A x, A y) { return x < y ? x : y; }
   __device__ static __forceinline__ void atomic(A* p, A v) { atomicMin(p, v); }
@@ -625,36 +625,31 @@ __device__ __forceinline__ int team_exclusive_scan(int x, int* scratch /* >= 33 
   return r;
 }
 
-// Exclusive scan of one int64 per thread across a CTA (blockDim.x threads,
-// a multiple of 32, at most 1024).  scratch: >= 33 long longs.
-__device__ __forceinline__ long long cta_exclusive_scan64(long long x, long long* scratch,
-                                                         long long& total) {
+// Exclusive scan of one int or int64 per thread across a CTA (blockDim.x
+// threads, a multiple of 32, at most 1024) with a single barrier: every warp
+// scans the warps' totals itself.  scratch: 32 values, free again after the
+// caller's next barrier.
+template <class T>
+__device__ __forceinline__ T cta_exclusive_scan(T x, T* scratch, T& total) {
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const int nw = blockDim.x >> 5;
-  long long incl = x;
+  T incl = x;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    long long y = __shfl_up_sync(0xffffffffu, incl, o);
+    const T y = __shfl_up_sync(0xffffffffu, incl, o);
     if (lane >= o) incl += y;
   }
   if (lane == 31) scratch[w] = incl;
   __syncthreads();
-  if (w == 0) {
-    long long v = lane < nw ? scratch[lane] : 0;
-    long long vi = v;
+  T t = lane < nw ? scratch[lane] : T(0);
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      long long y = __shfl_up_sync(0xffffffffu, vi, o);
-      if (lane >= o) vi += y;
-    }
-    if (lane < nw) scratch[lane] = vi - v;
-    if (lane == nw - 1) scratch[32] = vi;
+  for (int o = 1; o < 32; o <<= 1) {
+    const T y = __shfl_up_sync(0xffffffffu, t, o);
+    if (lane >= o) t += y;
   }
-  __syncthreads();
-  total = scratch[32];
-  const long long r = scratch[w] + incl - x;
-  __syncthreads();
-  return r;
+  total = __shfl_sync(0xffffffffu, t, 31);
+  const T before = __shfl_sync(0xffffffffu, t, (w + 31) & 31);  // the warps before this one
+  return (w ? before : T(0)) + incl - x;
 }
 
 // First index in the sorted run col[q0, q1) whose column is >= x (one thread).
@@ -725,7 +720,7 @@ struct NoValue {};
 // ms on R-MAT s18 and 21.7 instead of 14.9 on the block-clustered product).
 // The loop is bound by the instructions it issues, so a range's pieces are
 // walked in an inner loop on 32-bit offsets from its first entry.
-// All threads of the CTA must call it.
+// All threads of the CTA must call it; it ends with a barrier.
 struct PieceSmem {
   int* poff;        // [blockDim.x] first piece of each nonempty range (chunk numbering)
   long long* q0;    // [blockDim.x] first B entry of the range
@@ -769,7 +764,7 @@ __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B,
     const long long np = q0 < q1 ? (q1 - q0 + P - 1) / P : 0;
     // one scan numbers the pieces (high bits) and the nonempty ranges (low 11 bits)
     long long packed_total;
-    const long long packed = cta_exclusive_scan64((np << 11) | (np > 0 ? 1 : 0), sm.scan, packed_total);
+    const long long packed = cta_exclusive_scan((np << 11) | (np > 0 ? 1 : 0), sm.scan, packed_total);
     const long long npieces = packed_total >> 11;
     const int ne = (int)(packed_total & 2047);
     if (npieces >= (1 << 24)) {  // 2^31 products or more: 32-bit offsets do not do; entry by entry

@@ -342,7 +342,6 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
   // values need no copy out of a scratch slice; other 8-byte semirings use
   // the slice and convert on the way out.
   constexpr bool kInPlace = kL2 && kRankInPlace && (SR == 1 || SR == 2);
-  constexpr int WPT = kSpanWords / CTA;
   static_assert(WCAP <= 65535, "a window's entry counts are kept in 16 bits");
   extern __shared__ __align__(16) unsigned char rank_smem[];
   // shared layout: [(or,and) bits] [bx] [by] [4-byte accumulators] [iterator scratch];
@@ -359,8 +358,8 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
   unsigned short* by = reinterpret_cast<unsigned short*>(bx + kSpanWords);
   Acc* acc = nullptr;
   long long* bal = reinterpret_cast<long long*>(rank_smem + RankShape<SR>::kAccBytes + RankShape<SR>::kWordBytes);
-  __shared__ int scratch[33];
-  __shared__ long long scan64[33];
+  __shared__ int scratch[32];
+  __shared__ long long scan64[32];
   const PieceSmem sm(bal, CTA, scan64);
   __shared__ long long s_base;
   __shared__ long long next;
@@ -434,20 +433,22 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
                        const unsigned off = (unsigned)((int64_t)c - lo);
                        if (chk(off < 32u * (unsigned)nw, 36, c)) atomicOr(&bx[off >> 5], 1u << (off & 31));
                      });
-      __syncthreads();
     }
     // exclusive prefix of word popcounts
-    {
+    const auto rank_words = [&](auto wpt) {
+      constexpr int WPT = decltype(wpt)::value;
       int c[WPT];
       popc_words<WPT>(bx, tid * WPT, nw, c);
       int mine = 0;
 #pragma unroll
       for (int j = 0; j < WPT; ++j) mine += c[j];
       int total;
-      const int run = team_exclusive_scan<CTA>(mine, scratch, total);
-      store_counts<WPT>(by, tid * WPT, nw, run, c);
+      const int run = cta_exclusive_scan(mine, scratch, total);
+      if (tid * WPT < nw) store_counts<WPT>(by, tid * WPT, nw, run, c);
       if (tid == 0 && total != wd.count) flag_error(err, 23);
-    }
+    };
+    if (nw > 8 * CTA) rank_words(std::integral_constant<int, kSpanWords / CTA>{});
+    else rank_words(std::integral_constant<int, 8>{});
     __syncthreads();
     // pass 2: accumulate at the rank of each product's column: the entries of
     // the words before its word and the word's bits up to it, less itself
@@ -458,7 +459,10 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
                      const unsigned off = (unsigned)c - lo32;
                      if (!chk(off < 32u * (unsigned)nw, 36, c)) return;
                      const int slot = (int)by[off >> 5] + __popc(bx[off >> 5] << (~off & 31u)) - 1;
-                     if (guard((unsigned)slot < (unsigned)lim, 37, out + slot)) {
+                     // shared accumulators hold every entry of the bitmap, so a set bit's slot
+                     // is inside; C in place may end before (an inconsistent count)
+                     if (kInPlace ? guard((unsigned)slot < (unsigned)lim, 37, out + slot)
+                                  : chk((unsigned)slot < (unsigned)lim, 37, out + slot)) {
                        if constexpr (kInPlace) {
                          red_add_hint(&wacc[slot], S::mul(a_cur, bv), pol);
                        } else if constexpr (kBits) {
@@ -468,7 +472,6 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
                        }
                      }
                    });
-    __syncthreads();
     if (kInPlace && lim > 0) {  // the window is complete: its lines back to normal priority
       const uintptr_t b0 = reinterpret_cast<uintptr_t>(wacc) & ~(uintptr_t)127;
       const uintptr_t b1 = reinterpret_cast<uintptr_t>(wacc + lim);

@@ -72,11 +72,18 @@ __global__ void __launch_bounds__(CTA) k_sym_hash(DevCSR A, DevCSR B, const int3
   }
 }
 
+// Shape of the bitmap pass: four CTAs an SM, 32 registers.  Most of a row's
+// time is not its products (R-MAT s16: 27000 of them a row) but the scans,
+// barriers and window cuts around them, which smaller CTAs repeat in fewer
+// warps: 512 x 4 against 1024 x 2 threads took R-MAT s18 8.3 -> 7.4 ms, s16 1.61
+// -> 1.22, a merge of 8 parts 0.83 -> 0.60; 512 x 3 7.7 and 256 x 6 8.5 ms on s18.
+constexpr int kBmCta = 512, kBmPerSm = 4;
+
 // Heavy rows (u > 512): one CTA per (heavy row h, span) unit.  The bitmap
 // covers the span's columns [lo, hi); after counting, the span is cut into
 // rank windows (WinCut), appended to
 // `wins` (when non-null) for the numeric phase.  Units are taken from a queue.
-__global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, const int32_t* heavy_rows,
+__global__ void __launch_bounds__(kBmCta, kBmPerSm) k_sym_bitmap(DevCSR A, DevCSR B, const int32_t* heavy_rows,
                                                      int64_t n_heavy, int64_t spans,
                                                      const int64_t* flops, WinCut wcut, int64_t* nnz,
                                                      int32_t* span_counts, int2* span_wins,
@@ -84,13 +91,12 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
                                                      unsigned* hbits, int b_sorted,
                                                      int64_t* counters) {
   extern __shared__ __align__(16) unsigned sym_bm[];
-  __shared__ int scratch[33];
-  __shared__ long long scan64[33];
+  __shared__ int scratch[32];
+  __shared__ long long scan64[32];
   __shared__ int wstart[kMaxWindowsPerSpan];
   __shared__ int wrank[kMaxWindowsPerSpan];
   __shared__ long long wbase;
   __shared__ long long next;
-  constexpr int WPT = kSpanWords / 1024;  // bitmap words per thread in the scan
   const int tid = threadIdx.x;
   if (b_sorted < 0) {  // sizes on the device: heavy segment of perm, count, B's sortedness
     heavy_rows += counters[kCntSym + 1] + counters[kCntSym + 2] + counters[kCntSym + 3];
@@ -100,10 +106,10 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
   const int64_t units = n_heavy * spans;
   const int bm_words = (int)min((int64_t)kSpanWords, (B.ncols + 31) / 32);
   long long* bal = reinterpret_cast<long long*>(sym_bm + ((bm_words + 3) & ~3));
-  const PieceSmem sm(bal, 1024, scan64);
+  const PieceSmem sm(bal, kBmCta, scan64);
   // the bitmap starts clear; each unit clears the words it set once it has
   // read them, so no unit starts with a clearing pass of its own
-  for (int w = tid; w < bm_words; w += 1024) sym_bm[w] = 0u;
+  for (int w = tid; w < bm_words; w += kBmCta) sym_bm[w] = 0u;
   take_unit(counters + kSymQueue, &next);
   __syncthreads();
   for (int64_t u = next; u < units; u = next) {
@@ -128,26 +134,49 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
                      const unsigned off = (unsigned)c - lo32;
                      if (chk(off < 32u * (unsigned)nwords, 40, c)) atomicOr(&sym_bm[off >> 5], 1u << (off & 31));
                    });
-    __syncthreads();
-    if (hbits) {
-      unsigned* dst = hbits + (size_t)(h * spans + sp) * kSpanWords;
-      for (int w = tid; w < nwords; w += 1024) st_out(dst + w, sym_bm[w]);
-    }
-
-    // exclusive prefix of the word popcounts (WPT consecutive words per thread)
-    int c[WPT];
-    popc_words<WPT>(sym_bm, tid * WPT, nwords, c);
-    int mine = 0;
+    // The prefix of the word popcounts (WPT consecutive words per thread) cuts
+    // the span into windows: word w belongs to window floor(weight(w) / cut),
+    // where weight(w) = per_word * w + per_entry * (entries in words < w).  A
+    // word adds at most per_word + 32 * per_entry <= cut, so window indices
+    // run 0..K-1 without gaps and every window has a first word.
+    int total, K;
+    const auto cut_windows = [&](auto wpt) {
+      constexpr int WPT = decltype(wpt)::value;
+      const int w0 = tid * WPT;
+      int c[WPT];
+      popc_words<WPT>(sym_bm, w0, nwords, c);
+      int mine = 0;
 #pragma unroll
-    for (int j = 0; j < WPT; ++j) mine += c[j];
-    int total;
-    int run = team_exclusive_scan<1024>(mine, scratch, total);  // entries before my first word
-    // Windows: word w belongs to window floor(weight(w) / cut), where
-    // weight(w) = per_word * w + per_entry * (entries in words < w).  A word
-    // adds at most per_word + 32 * per_entry <= cut, so window indices run
-    // 0..K-1 without gaps and every window has a first word.
-    const int last = wcut.per_word * (nwords - 1) + wcut.per_entry * (total - __popc(sym_bm[nwords - 1]));
-    int K = (wins && total > 0) ? last / wcut.cut + 1 : 0;
+      for (int j = 0; j < WPT; ++j) mine += c[j];
+      int run = cta_exclusive_scan(mine, scratch, total);  // entries before my first word
+      const int last = wcut.per_word * (nwords - 1) + wcut.per_entry * (total - __popc(sym_bm[nwords - 1]));
+      K = (wins && total > 0) ? last / wcut.cut + 1 : 0;
+      if (K <= 1 || w0 >= nwords) return;
+      // kcur = the window of the word before the current one; one division
+      // per thread, then a comparison per word (a word crosses at most one
+      // multiple of cut)
+      int weight = wcut.per_word * w0 + wcut.per_entry * run;
+      int kcur = 0;
+      if (w0 > 0) kcur = (weight - wcut.per_word - wcut.per_entry * __popc(sym_bm[w0 - 1])) / wcut.cut;
+      int nextb = (kcur + 1) * wcut.cut;
+      if (weight + wcut.per_word * WPT + wcut.per_entry * mine < nextb) return;  // no cut among its words
+#pragma unroll
+      for (int j = 0; j < WPT; ++j) {
+        const int w = w0 + j;
+        if (w > 0 && w < nwords && weight >= nextb) {  // word w opens window kcur + 1
+          ++kcur;
+          nextb += wcut.cut;
+          if (kcur < K && kcur < kMaxWindowsPerSpan) {
+            wstart[kcur] = w;
+            wrank[kcur] = run;
+          }
+        }
+        run += c[j];
+        weight += wcut.per_word + wcut.per_entry * c[j];
+      }
+    };
+    if (nwords > 4 * kBmCta) cut_windows(std::integral_constant<int, kSpanWords / kBmCta>{});
+    else cut_windows(std::integral_constant<int, 4>{});
     if (K > kMaxWindowsPerSpan) {  // cut too small for this span width
       if (tid == 0) atomicCAS((unsigned long long*)&counters[kError], 0ull, 31ull);
       K = 0;
@@ -155,29 +184,6 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
     if (tid == 0) {
       wstart[0] = 0;
       wrank[0] = 0;
-    }
-    // kcur = the window of the word before the current one; one division
-    // per thread, then a comparison per word (a word crosses at most one
-    // multiple of cut)
-    int weight = wcut.per_word * tid * WPT + wcut.per_entry * run;
-    int kcur = 0, nextb = wcut.cut;
-    if (tid * WPT > 0 && tid * WPT < nwords) {
-      kcur = (weight - wcut.per_word - wcut.per_entry * __popc(sym_bm[tid * WPT - 1])) / wcut.cut;
-      nextb = (kcur + 1) * wcut.cut;
-    }
-#pragma unroll
-    for (int j = 0; j < WPT; ++j) {
-      const int w = tid * WPT + j;
-      if (w > 0 && w < nwords && weight >= nextb) {  // word w opens window kcur + 1
-        ++kcur;
-        nextb += wcut.cut;
-        if (kcur < K) {
-          wstart[kcur] = w;
-          wrank[kcur] = run;
-        }
-      }
-      run += c[j];
-      weight += wcut.per_word + wcut.per_entry * c[j];
     }
     if (tid == 0) {
       long long b = -1;
@@ -190,6 +196,10 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
       }
       wbase = b;
       if (span_wins) span_wins[h * spans + sp] = make_int2((int)(b >= 0 ? b : 0), b >= 0 ? K : 0);
+    }
+    if (hbits) {  // (the other warps, while the first one waits for its window base)
+      unsigned* dst = hbits + (size_t)(h * spans + sp) * kSpanWords;
+      for (int w = tid; w < nwords; w += kBmCta) st_out(dst + w, sym_bm[w]);
     }
     __syncthreads();
     if (tid < K && wbase >= 0) {
@@ -206,7 +216,7 @@ __global__ void __launch_bounds__(1024, 2) k_sym_bitmap(DevCSR A, DevCSR B, cons
       span_counts[h * spans + sp] = total;
       if (total) atomicAdd((unsigned long long*)&nnz[i], (unsigned long long)total);
     }
-    for (int w = tid; w < nwords; w += 1024) sym_bm[w] = 0u;  // every read of them is done
+    for (int w = tid; w < nwords; w += kBmCta) sym_bm[w] = 0u;  // every read of them is done
     take_unit(counters + kSymQueue, &next);
     __syncthreads();
   }
@@ -250,7 +260,7 @@ void launch_check_sorted(const DevCSR& B, int64_t* counters, cudaStream_t s, int
 void prepare_symbolic_dev() {
   constexpr int CTA = 512, TEAM = 512, TBL = 2 * kSymLargeMax;
   set_smem(k_sym_hash<CTA, TEAM, TBL>, TBL * sizeof(int));
-  set_smem(k_sym_bitmap, (size_t)kSpanWords * sizeof(unsigned) + 1024 * PieceSmem::kBytesPerThread);
+  set_smem(k_sym_bitmap, (size_t)kSpanWords * sizeof(unsigned) + kBmCta * PieceSmem::kBytesPerThread);
 }
 
 void launch_symbolic_dev(const DevCSR& A, const DevCSR& B, const int32_t* perm, int64_t* counters,
@@ -262,8 +272,8 @@ void launch_symbolic_dev(const DevCSR& A, const DevCSR& B, const int32_t* perm, 
     const int64_t spans = (B.ncols + kSpanCols - 1) / kSpanCols;
     const int64_t width = B.ncols < kSpanCols ? B.ncols : kSpanCols;
     const size_t bm_words = (size_t)((width + 31) / 32);
-    const size_t smem = ((bm_words + 3) & ~(size_t)3) * sizeof(unsigned) + 1024 * PieceSmem::kBytesPerThread;
-    k_sym_bitmap<<<sms * 2, 1024, smem, s>>>(A, B, perm, 0, spans, flops, wcut, nnz, span_counts,
+    const size_t smem = ((bm_words + 3) & ~(size_t)3) * sizeof(unsigned) + kBmCta * PieceSmem::kBytesPerThread;
+    k_sym_bitmap<<<sms * kBmPerSm, kBmCta, smem, s>>>(A, B, perm, 0, spans, flops, wcut, nnz, span_counts,
                                              span_wins, wins, win_cap, nullptr, -1, counters);
   }
   const int64_t* dc = counters + kCntSym;
@@ -317,9 +327,9 @@ void launch_symbolic(const DevCSR& A, const DevCSR& B, const int32_t* perm,
     const int64_t spans = (B.ncols + kSpanCols - 1) / kSpanCols;
     const int64_t width = B.ncols < kSpanCols ? B.ncols : kSpanCols;
     const size_t bm_words = (size_t)((width + 31) / 32);
-    const size_t smem = ((bm_words + 3) & ~(size_t)3) * sizeof(unsigned) + 1024 * PieceSmem::kBytesPerThread;
+    const size_t smem = ((bm_words + 3) & ~(size_t)3) * sizeof(unsigned) + kBmCta * PieceSmem::kBytesPerThread;
     set_smem(k_sym_bitmap, smem);
-    k_sym_bitmap<<<capped(seg_count[kSymHeavy] * spans, (int64_t)sms * 2), 1024, smem, s>>>(
+    k_sym_bitmap<<<capped(seg_count[kSymHeavy] * spans, (int64_t)sms * kBmPerSm), kBmCta, smem, s>>>(
         A, B, perm + seg_begin[kSymHeavy], seg_count[kSymHeavy], spans, flops, wcut, nnz,
         span_counts, span_wins, wins, win_cap, hbits, b_sorted, counters);
     ++*launches;
