@@ -20,8 +20,13 @@ struct StackPart {
   int32_t width;       // output width of the part's rows (k_i)
 };
 
-// blockIdx.y = part; x-blocks stride over the part's rows and entries.  The
-// last part also writes the closing row pointer.
+// blockIdx.y = part; x-blocks stride over the part's rows and entries, four
+// entries per thread in flight.  The last part also writes the closing row
+// pointer.  Parts differ in size by orders of magnitude, so a part gets enough
+// blocks for the largest to be copied at memory speed, and the blocks that a
+// small part leaves idle end at once (64 fp64 parts of 256 to 65536 rows, 8
+// blocks each and one entry in flight: 1.46 ms for 37M entries, 8x the copy's
+// time).
 template <class T>
 __global__ void __launch_bounds__(256) k_stack(const StackPart* parts, int nparts, int64_t* rp_out,
                                                int32_t* col_out, T* val_out, int32_t* rcols_out) {
@@ -36,9 +41,24 @@ __global__ void __launch_bounds__(256) k_stack(const StackPart* parts, int npart
   const int64_t nnz = pt.rp[pt.nrows] - base;
   if (t0 == 0 && (int)blockIdx.y == nparts - 1) rp_out[pt.row_off + pt.nrows] = pt.nnz_off + nnz;
   const T* src = static_cast<const T*>(pt.val) + base;
-  for (int64_t q = t0; q < nnz; q += stride) {
-    col_out[pt.nnz_off + q] = pt.col[base + q] + pt.col_add;
-    val_out[pt.nnz_off + q] = src[q];
+  const int32_t* csrc = pt.col + base;
+  int32_t* cdst = col_out + pt.nnz_off;
+  T* vdst = val_out + pt.nnz_off;
+  for (int64_t q = t0; q < nnz; q += 4 * stride) {
+    int32_t c[4];
+    T v[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (q + u * stride < nnz) {
+        c[u] = __ldcs(csrc + q + u * stride);
+        v[u] = __ldcs(src + q + u * stride);
+      }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+      if (q + u * stride < nnz) {
+        cdst[q + u * stride] = c[u] + pt.col_add;
+        vdst[q + u * stride] = v[u];
+      }
   }
 }
 
@@ -221,7 +241,8 @@ void launch_merge_selector(int64_t m, int k, int vsz, uint64_t one_bits, int64_t
 void launch_stack(const void* parts_dev, int nparts, int vsz, int64_t* rp_out, int32_t* col_out,
                   void* val_out, int32_t* rcols_out, cudaStream_t s, int sms) {
   if (nparts <= 0) return;
-  dim3 grid((unsigned)(nparts < 64 ? sms * 4 : 8), (unsigned)nparts);
+  const int per_part = sms * 32 / nparts;
+  dim3 grid((unsigned)(per_part < 8 ? 8 : per_part > sms * 8 ? sms * 8 : per_part), (unsigned)nparts);
   const StackPart* pp = static_cast<const StackPart*>(parts_dev);
   switch (vsz) {
     case 8: k_stack<uint64_t><<<grid, 256, 0, s>>>(pp, nparts, rp_out, col_out, static_cast<uint64_t*>(val_out), rcols_out); break;

@@ -395,8 +395,8 @@ __device__ __forceinline__ void for_bitmap_columns(const unsigned* bits, const u
   }
 }
 
-// The columns of a window's cnt entries, col0 + offset, to out[0 .. min(cnt,
-// lim)) through a shared buffer of cnt words: the bitmap is walked a word per
+// The columns of a window's cnt entries, col0 + offset, to out[0 .. lim)
+// (lim <= cnt) through a shared buffer of cnt words: the bitmap is walked a word per
 // thread into the buffer, and the buffer copied out coalesced.  All threads of
 // the CTA call it, after a barrier.  (u32 numeric of R-MAT s18 35.6 -> 34.0 ms
 // against one L2 request per entry.  Where no shared memory of that size is
@@ -404,7 +404,7 @@ __device__ __forceinline__ void for_bitmap_columns(const unsigned* bits, const u
 // (or,and): those windows use for_bitmap_columns.)
 template <int CTA>
 __device__ __forceinline__ void write_columns(const unsigned* bits, const unsigned short* pre, int nw, int cnt,
-                                              int64_t lim, int32_t col0, int32_t* buf, int32_t* out) {
+                                              int lim, int32_t col0, int32_t* buf, int32_t* out) {
   const int tid = threadIdx.x;
   for (int w = tid; w < nw; w += CTA) {
     unsigned word = bits[w];
@@ -417,8 +417,8 @@ __device__ __forceinline__ void write_columns(const unsigned* bits, const unsign
     }
   }
   __syncthreads();
-  for (int t = tid; t < cnt; t += CTA)
-    if (guard(t < lim, 39, t)) st_out(out + t, buf[t]);
+#pragma unroll 4
+  for (int t = tid; t < lim; t += CTA) st_out(out + t, buf[t]);
 }
 
 enum SymTier { kSymEmpty = 0, kSymWarp = 1, kSymSmall = 2, kSymLarge = 3, kSymHeavy = 4, kSymTiers = 5 };

@@ -480,18 +480,19 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
     }
     // write the window: values by slot (coalesced; in place they are there
     // already), columns by word
+    const int n_out = (int)max((int64_t)0, min((int64_t)cnt, row_end - out));
+    guard(n_out == cnt, 38, row_end);
     if constexpr (kBits) {
-      for (int t = tid; t < cnt; t += CTA)
-        if (guard(out + t < row_end, 38, out + t))
-          st_out(Cval + out + t, (TC)((accbits[t >> 5] >> (t & 31)) & 1u));
+      for (int t = tid; t < n_out; t += CTA)
+        st_out(Cval + out + t, (TC)((accbits[t >> 5] >> (t & 31)) & 1u));
     } else if constexpr (!kInPlace) {
-      for (int t = tid; t < cnt; t += CTA)
-        if (guard(out + t < row_end, 38, out + t))
-          st_out(Cval + out + t, S::out(kL2 ? __ldcg(wacc + t) : wacc[t]));
+      TC* const ov = Cval + out;
+#pragma unroll 4
+      for (int t = tid; t < n_out; t += CTA) st_out(ov + t, S::out(kL2 ? __ldcg(wacc + t) : wacc[t]));
     }
     if constexpr (kPool) {  // the accumulators are free once the values are out
       __syncthreads();
-      write_columns<CTA>(bx, by, nw, cnt, row_end - out, (int32_t)lo, reinterpret_cast<int32_t*>(acc), Ccol + out);
+      write_columns<CTA>(bx, by, nw, cnt, n_out, (int32_t)lo, reinterpret_cast<int32_t*>(acc), Ccol + out);
     } else {
       for_bitmap_columns<kL2 ? kDenseWordBits : 0, CTA>(bx, by, nw, cnt, [&](int j, int c) {
         const int64_t o = out + j;
