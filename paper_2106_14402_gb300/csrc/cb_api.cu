@@ -10,8 +10,10 @@
 #include <atomic>
 #include <deque>
 #include <memory>
+#include <mutex>
 #include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -103,6 +105,47 @@ constexpr size_t kIdleShare = 4;
 constexpr size_t kIdleUnchecked = size_t(1) << 30;
 constexpr size_t kIdleMoved = size_t(64) << 20;  // reading the pool's counters costs 20 us in flight
 
+// Pools of contexts that are gone, for later contexts of their device: trimmed
+// to what results still hold, and never destroyed (a pool destroyed under a
+// result that outlives its context is the likely cause of a crash in a later
+// memory call).
+struct PoolList {
+  std::mutex lock;
+  std::vector<std::pair<int, cudaMemPool_t>> idle;  // device, pool
+};
+PoolList& pool_list() {
+  static PoolList* const list = new PoolList;  // outlives every context
+  return *list;
+}
+
+void retire_pool(cb_ctx* ctx) {
+  if (!ctx->pool) return;
+  uint64_t hold = 0;
+  const bool ok = cudaStreamSynchronize(ctx->stream) == cudaSuccess &&
+                  cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &hold) == cudaSuccess &&
+                  cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess;
+  if (ok) {
+    PoolList& l = pool_list();
+    const std::lock_guard<std::mutex> guard(l.lock);
+    l.idle.emplace_back(ctx->device, ctx->pool);
+  }
+  ctx->pool = nullptr;
+}
+
+cudaMemPool_t reuse_pool(int device) {
+  PoolList& l = pool_list();
+  const std::lock_guard<std::mutex> guard(l.lock);
+  for (size_t k = l.idle.size(); k-- > 0;) {
+    if (l.idle[k].first != device) continue;
+    const cudaMemPool_t p = l.idle[k].second;
+    l.idle.erase(l.idle.begin() + (std::ptrdiff_t)k);
+    uint64_t used = 0;
+    if (cudaMemPoolGetAttribute(p, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess) return p;
+    (void)cudaGetLastError();  // the device was reset since
+  }
+  return nullptr;
+}
+
 cudaError_t ensure_pool(cb_ctx* ctx) {
   if (ctx->pool || !ctx->pooled) return cudaSuccess;
   cudaMemPoolProps props = {};
@@ -111,7 +154,7 @@ cudaError_t ensure_pool(cb_ctx* ctx) {
   props.location.id = ctx->device;
   cudaDeviceProp dp;
   cudaError_t e = cudaGetDeviceProperties(&dp, ctx->device);
-  if (e == cudaSuccess) e = cudaMemPoolCreate(&ctx->pool, &props);
+  if (e == cudaSuccess && !(ctx->pool = reuse_pool(ctx->device))) e = cudaMemPoolCreate(&ctx->pool, &props);
   if (e != cudaSuccess) {
     ctx->pool = nullptr;
     return e;
@@ -1668,8 +1711,7 @@ void cb_ctx_destroy(cb_ctx* ctx) {
   if (ctx->spa_bits) cudaFree(ctx->spa_bits);
   for (cudaEvent_t e : ctx->ev)
     if (e) cudaEventDestroy(e);
-  // arrays of C still in use keep their part of the pool until they are freed
-  if (ctx->pool) cudaMemPoolDestroy(ctx->pool);
+  retire_pool(ctx);  // arrays of C still in use keep their part of it until they are freed
   delete ctx;
 }
 
