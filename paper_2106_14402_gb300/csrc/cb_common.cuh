@@ -699,7 +699,7 @@ __device__ __forceinline__ void row_slice(const DevCSR& B, const SplitTable& t, 
   s1 = b0;
 }
 
-// Marks a call of for_row_pieces that needs no values of B.
+// Marks a call of for_row_pieces that needs no values of A or B.
 struct NoValue {};
 
 // All products of row i whose columns lie in [lo, hi), for a whole CTA: the
@@ -709,10 +709,10 @@ struct NoValue {};
 // pieces are numbered by one CTA scan, and every warp takes an equal
 // contiguous run of pieces.  Inside a piece the A entry is the same for the
 // whole warp.
-//   on_entry(p): called (warp-uniformly) when the warp reaches the pieces of
-//                A entry p; returns a token (e.g. A's value) for them;
-//   f(t, c, v):  one product: the token, column c and B's value there (values
-//                from Bval; V = NoValue reads none).
+//   f(a, c, v):  one product: A's value (from Aval), column c and B's value
+//                there (from Bval); of type NoValue they are not read.
+// A's values come with the ranges, through shared memory: read by the warp that
+// reaches a range they cost it a load's latency there.
 // Lane l takes entries l, l + 32, l + 64, l + 96 of a piece: coalesced loads,
 // all in flight before the callbacks, and neighbouring lanes meet neighbouring
 // columns, whose accumulators often share an L2 sector (with four consecutive
@@ -721,28 +721,30 @@ struct NoValue {};
 // The loop is bound by the instructions it issues, so a range's pieces are
 // walked in an inner loop on 32-bit offsets from its first entry.
 // All threads of the CTA must call it; it ends with a barrier.
+template <class T>  // A's value type, or NoValue
 struct PieceSmem {
-  int* poff;        // [blockDim.x] first piece of each nonempty range (chunk numbering)
+  static constexpr bool kA = !std::is_same<T, NoValue>::value;
   long long* q0;    // [blockDim.x] first B entry of the range
+  T* a;             // [blockDim.x] A's value
   int* len;         // [blockDim.x] entries in the range
-  int* pa;          // [blockDim.x] A entry of the range (relative to the chunk)
-  long long* scan;  // [33]
-  static constexpr size_t kBytesPerThread = sizeof(long long) + 3 * sizeof(int);
+  int* poff;        // [blockDim.x] first piece of each nonempty range (chunk numbering)
+  long long* scan;  // [32]
+  static constexpr size_t kBytesPerThread = sizeof(long long) + 2 * sizeof(int) + (kA ? sizeof(T) < 4 ? 4 : sizeof(T) : 0);
   // carved from threads * kBytesPerThread bytes, 8-byte aligned
   __device__ PieceSmem(void* p, int threads, long long* scan_) : scan(scan_) {
     q0 = static_cast<long long*>(p);
     len = reinterpret_cast<int*>(q0 + threads);
     poff = len + threads;
-    pa = poff + threads;
+    a = reinterpret_cast<T*>(poff + threads);
   }
 };
 
-template <class V, class FA, class F>
+template <class T, class V, class F>
 __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B, const SplitTable& tab,
                                                int64_t i, int64_t lo, int64_t hi, bool whole, bool sorted,
-                                               const PieceSmem& sm, const V* Bval, FA&& on_entry, F&& f) {
+                                               const PieceSmem<T>& sm, const T* Aval, const V* Bval, F&& f) {
   constexpr int P = 128;
-  constexpr bool kVals = !std::is_same<V, NoValue>::value;
+  constexpr bool kVals = !std::is_same<V, NoValue>::value, kA = PieceSmem<T>::kA;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const int nthr = blockDim.x, nwarp = nthr >> 5;
   const int64_t a0 = A.rp[i], a1 = A.rp[i + 1];
@@ -752,8 +754,10 @@ __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B,
   for (int64_t c0 = a0; c0 < a1; c0 += nthr) {
     const int nch = (int)min((int64_t)nthr, a1 - c0);
     int64_t q0 = 0, q1 = 0;
+    T av{};
     if (tid < nch) {
       const int k = A.col[c0 + tid];
+      if constexpr (kA) av = ldg_val(Aval + c0 + tid);
       if (!whole && sorted) {
         row_slice(B, tab, k, lo, hi, q0, q1);
       } else {
@@ -772,9 +776,11 @@ __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B,
         if (tid == t) {
           sm.q0[0] = q0;
           sm.q0[1] = q1;
+          if constexpr (kA) sm.a[0] = av;
         }
         __syncthreads();
-        const auto tok = on_entry(c0 + t);
+        T tok{};
+        if constexpr (kA) tok = sm.a[0];
         const int64_t end = sm.q0[1];
         for (int64_t q = sm.q0[0] + tid; q < end; q += nthr) {
           const int c = __ldg(B.col + q);
@@ -789,9 +795,9 @@ __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B,
     if (np > 0) {
       const int slot = (int)(packed & 2047);
       sm.poff[slot] = (int)(packed >> 11);
+      if constexpr (kA) sm.a[slot] = av;
       sm.q0[slot] = q0;
       sm.len[slot] = (int)(q1 - q0);
-      sm.pa[slot] = tid;
     }
     __syncthreads();
     // equal runs of pieces per warp; nwarp is a power of two (512- and
@@ -810,7 +816,8 @@ __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B,
         const int len = sm.len[j];
         const int32_t* cp = B.col + sm.q0[j] + lane;
         const V* vp = kVals ? Bval + sm.q0[j] + lane : nullptr;
-        const auto tok = on_entry(c0 + sm.pa[j]);
+        T tok{};
+        if constexpr (kA) tok = sm.a[j];
         for (; left > 0 && s < len; --left, s += P) {
           int c[4];
           V v[4];

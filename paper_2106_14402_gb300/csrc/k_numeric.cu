@@ -270,13 +270,15 @@ constexpr bool kRankInPlace = true;
 //     ms together with the split table, 36.8 without it.)
 template <int SR>
 struct RankShape {
+  // what a product needs of its A entry
+  typedef typename std::conditional<Sem<SR>::kUsesA, typename Sem<SR>::TA, NoValue>::type Entry;
   static constexpr bool kBits = SR == 4;
   static constexpr bool kPool = !NumLimits<SR>::kL2Acc && !kBits;
   static constexpr int kCta = 512, kPerSm = 3;
   static constexpr size_t kAccBytes = kBits ? (size_t)NumLimits<SR>::kWcap / 8 : 0;
   static constexpr size_t kWordBytes =
       kPool ? (size_t)kWinPool : kSpanWords * (sizeof(unsigned) + sizeof(unsigned short));
-  static constexpr size_t kSmem = kAccBytes + kWordBytes + (size_t)kCta * PieceSmem::kBytesPerThread;
+  static constexpr size_t kSmem = kAccBytes + kWordBytes + (size_t)kCta * PieceSmem<Entry>::kBytesPerThread;
   // entries: kWcap less the words the last one may overshoot by; pool: less a
   // word's weight and the rounding of the words to 8
   static constexpr WinCut kCut =
@@ -360,7 +362,9 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
   long long* bal = reinterpret_cast<long long*>(rank_smem + RankShape<SR>::kAccBytes + RankShape<SR>::kWordBytes);
   __shared__ int scratch[32];
   __shared__ long long scan64[32];
-  const PieceSmem sm(bal, CTA, scan64);
+  typedef typename RankShape<SR>::Entry Entry;
+  const PieceSmem<Entry> sm(bal, CTA, scan64);
+  const Entry* const entries = reinterpret_cast<const Entry*>(A.val);
   __shared__ long long s_base;
   __shared__ long long next;
   const int tid = threadIdx.x, lane = tid & 31;
@@ -428,8 +432,8 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
     }
 
     if (!hbits) {  // pass 1: rebuild the window's columns
-      for_row_pieces(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, (const NoValue*)nullptr,
-                     [](int64_t) { return 0; }, [&](int, int c, NoValue) {
+      for_row_pieces(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, entries, (const NoValue*)nullptr,
+                     [&](Entry, int c, NoValue) {
                        const unsigned off = (unsigned)((int64_t)c - lo);
                        if (chk(off < 32u * (unsigned)nw, 36, c)) atomicOr(&bx[off >> 5], 1u << (off & 31));
                      });
@@ -453,9 +457,10 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
     // pass 2: accumulate at the rank of each product's column: the entries of
     // the words before its word and the word's bits up to it, less itself
     const unsigned lo32 = (unsigned)lo;
-    for_row_pieces(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, Bval,
-                   [&](int64_t p) { return S::kUsesA ? ldg_val(Aval + p) : TA(); },
-                   [&](TA a_cur, int c, TB bv) {
+    for_row_pieces(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, entries, Bval,
+                   [&](Entry entry, int c, TB bv) {
+                     TA a_cur{};
+                     if constexpr (S::kUsesA) a_cur = entry;
                      const unsigned off = (unsigned)c - lo32;
                      if (!chk(off < 32u * (unsigned)nw, 36, c)) return;
                      const int slot = (int)by[off >> 5] + __popc(bx[off >> 5] << (~off & 31u)) - 1;

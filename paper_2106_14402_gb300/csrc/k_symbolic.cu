@@ -106,7 +106,7 @@ __global__ void __launch_bounds__(kBmCta, kBmPerSm) k_sym_bitmap(DevCSR A, DevCS
   const int64_t units = n_heavy * spans;
   const int bm_words = (int)min((int64_t)kSpanWords, (B.ncols + 31) / 32);
   long long* bal = reinterpret_cast<long long*>(sym_bm + ((bm_words + 3) & ~3));
-  const PieceSmem sm(bal, kBmCta, scan64);
+  const PieceSmem<NoValue> sm(bal, kBmCta, scan64);
   // the bitmap starts clear; each unit clears the words it set once it has
   // read them, so no unit starts with a clearing pass of its own
   for (int w = tid; w < bm_words; w += kBmCta) sym_bm[w] = 0u;
@@ -130,7 +130,7 @@ __global__ void __launch_bounds__(kBmCta, kBmPerSm) k_sym_bitmap(DevCSR A, DevCS
     const int nwords = (int)((hi - lo + 31) / 32);
     const unsigned lo32 = (unsigned)lo;
     for_row_pieces(A, B, SplitTable{}, i, lo, hi, spans == 1 && !B.filter, b_sorted != 0, sm,
-                   (const NoValue*)nullptr, [](int64_t) { return 0; }, [&](int, int c, NoValue) {
+                   (const NoValue*)nullptr, (const NoValue*)nullptr, [&](NoValue, int c, NoValue) {
                      const unsigned off = (unsigned)c - lo32;
                      if (chk(off < 32u * (unsigned)nwords, 40, c)) atomicOr(&sym_bm[off >> 5], 1u << (off & 31));
                    });
@@ -260,7 +260,7 @@ void launch_check_sorted(const DevCSR& B, int64_t* counters, cudaStream_t s, int
 void prepare_symbolic_dev() {
   constexpr int CTA = 512, TEAM = 512, TBL = 2 * kSymLargeMax;
   set_smem(k_sym_hash<CTA, TEAM, TBL>, TBL * sizeof(int));
-  set_smem(k_sym_bitmap, (size_t)kSpanWords * sizeof(unsigned) + kBmCta * PieceSmem::kBytesPerThread);
+  set_smem(k_sym_bitmap, (size_t)kSpanWords * sizeof(unsigned) + kBmCta * PieceSmem<NoValue>::kBytesPerThread);
 }
 
 void launch_symbolic_dev(const DevCSR& A, const DevCSR& B, const int32_t* perm, int64_t* counters,
@@ -272,7 +272,7 @@ void launch_symbolic_dev(const DevCSR& A, const DevCSR& B, const int32_t* perm, 
     const int64_t spans = (B.ncols + kSpanCols - 1) / kSpanCols;
     const int64_t width = B.ncols < kSpanCols ? B.ncols : kSpanCols;
     const size_t bm_words = (size_t)((width + 31) / 32);
-    const size_t smem = ((bm_words + 3) & ~(size_t)3) * sizeof(unsigned) + kBmCta * PieceSmem::kBytesPerThread;
+    const size_t smem = ((bm_words + 3) & ~(size_t)3) * sizeof(unsigned) + kBmCta * PieceSmem<NoValue>::kBytesPerThread;
     k_sym_bitmap<<<sms * kBmPerSm, kBmCta, smem, s>>>(A, B, perm, 0, spans, flops, wcut, nnz, span_counts,
                                              span_wins, wins, win_cap, nullptr, -1, counters);
   }
@@ -327,7 +327,7 @@ void launch_symbolic(const DevCSR& A, const DevCSR& B, const int32_t* perm,
     const int64_t spans = (B.ncols + kSpanCols - 1) / kSpanCols;
     const int64_t width = B.ncols < kSpanCols ? B.ncols : kSpanCols;
     const size_t bm_words = (size_t)((width + 31) / 32);
-    const size_t smem = ((bm_words + 3) & ~(size_t)3) * sizeof(unsigned) + kBmCta * PieceSmem::kBytesPerThread;
+    const size_t smem = ((bm_words + 3) & ~(size_t)3) * sizeof(unsigned) + kBmCta * PieceSmem<NoValue>::kBytesPerThread;
     set_smem(k_sym_bitmap, smem);
     k_sym_bitmap<<<capped(seg_count[kSymHeavy] * spans, (int64_t)sms * kBmPerSm), kBmCta, smem, s>>>(
         A, B, perm + seg_begin[kSymHeavy], seg_count[kSymHeavy], spans, flops, wcut, nnz,
