@@ -2075,7 +2075,10 @@ int cb_spmspv(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_spvec* x, c
       y->idx = nullptr;
       y->val = nullptr;
     }
-    if (opt.validate) {
+    // the dense form queues the validation with the product: no chunk of A is
+    // pushed when it fails
+    const bool queued = opt.validate && n > 0 && nx > 0 && !(opt.flags & CB_FLAG_SPMSPV_BUCKET);
+    if (opt.validate && !queued) {
       ensure(ctx, &ctx->ws, &ctx->ws_cap, align_up(sizeof(int64_t) * cb::kCounters));
       int64_t* counters = static_cast<int64_t*>(ctx->ws);
       CB_CUDA(cudaMemsetAsync(counters, 0, sizeof(int64_t) * cb::kCounters, ctx->stream));
@@ -2104,7 +2107,7 @@ int cb_spmspv(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_spvec* x, c
       CB_CUDA(cudaMemsetAsync(ctx->spa_bits, 0, 4 * (size_t)nw, ctx->stream));
       ctx->spa_n = n;
     }
-    const DevCSR dA = dev(A);
+    DevCSR dA = dev(A);
     if (ctx->spa_sr != (int)sr) {
       cb::launch_spmspv_step((int)sr, 0, dA, nullptr, nullptr, 0, nullptr, nullptr, ctx->spa, nullptr,
                              ctx->spa_n, nullptr, nullptr, nullptr, nullptr, 0, nullptr, ctx->stream,
@@ -2125,6 +2128,10 @@ int cb_spmspv(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_spvec* x, c
     int64_t* wpre = cv.take<int64_t>(nw + 1);
     int64_t* partial = cv.take<int64_t>(cb::scan_partials(big));
     CB_CUDA(cudaMemsetAsync(counters, 0, sizeof(int64_t) * cb::kCounters, ctx->stream));
+    if (queued) {  // its error words: two of the tier cursors, unused here
+      cb::launch_validate(dA, A->nnz, 0, counters + cb::kCurNum, ctx->stream, ctx->sms);
+      dA.gate = counters + cb::kCurNum;
+    }
     mark(ctx, opt, 0);
     cb::launch_spmspv_step((int)sr, 1, dA, x->idx, x->val, nx, chunks, nullptr, nullptr, nullptr, n,
                            nullptr, nullptr, nullptr, nullptr, 0, counters + cb::kError, ctx->stream,
@@ -2139,6 +2146,7 @@ int cb_spmspv(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_spvec* x, c
     ctx->stats.kernels += 6;
     mark(ctx, opt, 1);
     read_counters(ctx, counters, wpre + nw, 1);
+    if (queued && ctx->host[cb::kCurNum]) fail(ctx, CB_ERR_INDEX, "A has invalid CSR index data");
     const int64_t total = ctx->host[cb::kCounters];
     const bool bad_x = ctx->host[cb::kError] != 0;
     int64_t cap = caller_buf ? opt.out_capacity : total;

@@ -38,8 +38,13 @@ constexpr int kChunk = 256;
 // K1.  An index outside [0, A.nrows) gets no chunks and sets *err.
 __global__ void __launch_bounds__(256) k_spmspv_chunks(DevCSR A, const int32_t* x_idx, int64_t nx,
                                                       int64_t* chunks, int64_t* err) {
+  const bool none = gated(A.gate);  // A is invalid: no chunk of it is read
   for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < nx;
        p += (int64_t)gridDim.x * blockDim.x) {
+    if (none) {
+      chunks[p] = 0;
+      continue;
+    }
     const int i = x_idx[p];
     if (i < 0 || (int64_t)i >= A.nrows) {
       chunks[p] = 0;
