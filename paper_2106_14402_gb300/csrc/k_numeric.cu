@@ -270,8 +270,12 @@ constexpr bool kRankInPlace = true;
 //     ms together with the split table, 36.8 without it.)
 template <int SR>
 struct RankShape {
-  // what a product needs of its A entry
-  typedef typename std::conditional<Sem<SR>::kUsesA, typename Sem<SR>::TA, NoValue>::type Entry;
+  // what a product needs of its A entry: the bits of its value (an integer, so
+  // that a signaling NaN weight passes through shared memory as it is)
+  typedef typename Sem<SR>::TA TA;
+  typedef typename std::conditional<
+      !Sem<SR>::kUsesA, NoValue,
+      typename std::conditional<std::is_same<TA, float>::value, unsigned, TA>::type>::type Entry;
   static constexpr bool kBits = SR == 4;
   static constexpr bool kPool = !NumLimits<SR>::kL2Acc && !kBits;
   static constexpr int kCta = 512, kPerSm = 3;
@@ -460,7 +464,7 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
     for_row_pieces(A, B, tab, i, lo, hi, whole, b_sorted != 0, sm, entries, Bval,
                    [&](Entry entry, int c, TB bv) {
                      TA a_cur{};
-                     if constexpr (S::kUsesA) a_cur = entry;
+                     if constexpr (S::kUsesA) memcpy(&a_cur, &entry, sizeof a_cur);
                      const unsigned off = (unsigned)c - lo32;
                      if (!chk(off < 32u * (unsigned)nw, 36, c)) return;
                      const int slot = (int)by[off >> 5] + __popc(bx[off >> 5] << (~off & 31u)) - 1;
