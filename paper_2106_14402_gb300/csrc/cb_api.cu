@@ -9,11 +9,11 @@
 #include <algorithm>
 #include <atomic>
 #include <deque>
+#include <map>
 #include <memory>
 #include <mutex>
 #include <new>
 #include <string>
-#include <utility>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -22,14 +22,23 @@
 #include "cb_common.cuh"
 #include "cb_kernels.h"
 
+namespace cb {
+// The library's memory pool of one device, shared by its contexts.
+struct DevicePool {
+  std::mutex lock;               // guards the members and the pool's threshold
+  cudaMemPool_t pool = nullptr;
+  int contexts = 0;              // contexts that allocate from it
+  size_t total = 0;              // the device's memory
+  std::atomic<size_t> moved{0};  // bytes taken and returned since the bound was set
+};
+}  // namespace cb
+
 struct cb_ctx {
   cudaStream_t stream = nullptr;
   int device = 0;
   int sms = 0;
-  bool pooled = true;   // allocate from a pool of its own (false: the device's default pool)
-  cudaMemPool_t pool = nullptr;
-  size_t pool_idle_max = 0;  // most idle memory the pool holds
-  std::atomic<size_t> pool_moved{0};  // bytes taken from and returned to the pool since its bound was set
+  bool pooled = true;   // allocate from the library's pool (false: the device's default pool)
+  cb::DevicePool* pool = nullptr;  // that pool, from the first allocation on
   void* ws = nullptr;   // workspace for per-row arrays
   size_t ws_cap = 0;
   void* ws2 = nullptr;  // workspace for heavy-row slice arrays
@@ -91,96 +100,137 @@ bool injected_alloc_failure(cb_ctx* ctx) {
   return true;
 }
 
-// The context's own pool.  The device's default pool returns everything free
-// to the system at each synchronisation, and a call synchronises before it
-// sizes C: mapping 1 GB took 0.85 ms and unmapping it 1.4 ms, a third of an
-// R-MAT s18 product (C of 35 GB) and half of a batched call.  This pool keeps
-// up to a quarter of the device's memory idle for the next call, but never
-// more than half of what is free beside it (bound_idle); it gives
-// everything back when the context goes, and when an allocation of its own
-// fails.  (R-MAT s18 products whose results live on for two calls: f64 94 ->
-// 56 ms, u32 74 -> 40; merge of 8 parts 10.4 -> 4.1; an ER product of 16384
-// rows 176 -> 91 us.)
+// The library's pool of a device.  The device's default pool returns
+// everything free to the system at each synchronisation, and a call
+// synchronises before it sizes C: mapping 1 GB took 0.85 ms and unmapping it
+// 1.4 ms, a third of an R-MAT s18 product (C of 35 GB) and half of a batched
+// call.  This pool keeps up to a quarter of the device's memory idle for the
+// next call, but never more than half of what is free beside it (or
+// kIdleUnchecked): set_bound, at the end of a call and whenever C is freed, by
+// whichever function and whichever context, which is why a device has one pool
+// for all contexts.  When a context goes, all idle memory goes back to the
+// system.  (Other allocations of the process get idle memory anyway: the
+// driver takes it back when it has nothing else.)  R-MAT s18 products whose
+// results live on for two calls: f64 94 -> 56 ms, u32 74 -> 40; merge of 8
+// parts 10.4 -> 4.1; an ER product of 16384 rows 176 -> 91 us.
 constexpr size_t kIdleShare = 4;
 constexpr size_t kIdleUnchecked = size_t(1) << 30;
-constexpr size_t kIdleMoved = size_t(64) << 20;  // reading the pool's counters costs 20 us in flight
+constexpr size_t kIdleMoved = size_t(64) << 20;  // between two settings of the bound
 
-// Pools of contexts that are gone, for later contexts of their device: trimmed
-// to what results still hold, and never destroyed (a pool destroyed under a
-// result that outlives its context is the likely cause of a crash in a later
-// memory call).
-struct PoolList {
-  std::mutex lock;
-  std::vector<std::pair<int, cudaMemPool_t>> idle;  // device, pool
+// Makes a device current for a scope.
+struct OnDevice {
+  int before = -1;
+  explicit OnDevice(int device) {
+    int now = -1;
+    if (cudaGetDevice(&now) == cudaSuccess && now != device && cudaSetDevice(device) == cudaSuccess) before = now;
+  }
+  ~OnDevice() {
+    if (before >= 0) cudaSetDevice(before);
+  }
 };
-PoolList& pool_list() {
-  static PoolList* const list = new PoolList;  // outlives every context
-  return *list;
+
+// Pools live as long as the process, so none is destroyed under a result that
+// outlives every context.
+cb::DevicePool& device_pool(int device) {
+  static std::mutex* const lock = new std::mutex;
+  static auto* const pools = new std::map<int, cb::DevicePool>;
+  const std::lock_guard<std::mutex> guard(*lock);
+  return (*pools)[device];
 }
 
-void retire_pool(cb_ctx* ctx) {
-  if (!ctx->pool) return;
-  uint64_t hold = 0;
-  const bool ok = cudaStreamSynchronize(ctx->stream) == cudaSuccess &&
-                  cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &hold) == cudaSuccess &&
-                  cudaMemPoolTrimTo(ctx->pool, 0) == cudaSuccess;
-  if (ok) {
-    PoolList& l = pool_list();
-    const std::lock_guard<std::mutex> guard(l.lock);
-    l.idle.emplace_back(ctx->device, ctx->pool);
+// Sets the pool's release threshold (its lock is held).  It covers what is in
+// use now and the idle memory allowed beside it; memory above it is returned
+// at the next synchronisation, or `now`.  (A stream-ordered free counts as idle
+// at once, while it is pending too.)  Takes half a microsecond a counter and 9
+// for the device's free memory, read only when more than kIdleUnchecked is idle.
+void set_bound(cb::DevicePool& p, int device, bool now = false) {
+  uint64_t used = 0, reserved = 0;
+  if (cudaMemPoolGetAttribute(p.pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess ||
+      cudaMemPoolGetAttribute(p.pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess) {
+    (void)cudaGetLastError();
+    return;
   }
-  ctx->pool = nullptr;
+  uint64_t idle = p.contexts ? p.total / kIdleShare : 0;
+  size_t free_b = 0, total_b = 0;
+  if (idle && reserved > used + kIdleUnchecked) {
+    const OnDevice on(device);
+    if (cudaMemGetInfo(&free_b, &total_b) == cudaSuccess)
+      idle = std::min<uint64_t>(idle, std::max<uint64_t>(free_b / 2, kIdleUnchecked));
+  }
+  uint64_t hold = used + idle;
+  cudaMemPoolSetAttribute(p.pool, cudaMemPoolAttrReleaseThreshold, &hold);
+  if (now) cudaMemPoolTrimTo(p.pool, hold);
+  p.moved = 0;
 }
 
-cudaMemPool_t reuse_pool(int device) {
-  PoolList& l = pool_list();
-  const std::lock_guard<std::mutex> guard(l.lock);
-  for (size_t k = l.idle.size(); k-- > 0;) {
-    if (l.idle[k].first != device) continue;
-    const cudaMemPool_t p = l.idle[k].second;
-    l.idle.erase(l.idle.begin() + (std::ptrdiff_t)k);
-    uint64_t used = 0;
-    if (cudaMemPoolGetAttribute(p, cudaMemPoolAttrUsedMemCurrent, &used) == cudaSuccess) return p;
-    (void)cudaGetLastError();  // the device was reset since
-  }
-  return nullptr;
+// Gives the pool's idle memory beyond `keep` bytes back to the system.
+cudaError_t give_back(cb::DevicePool& p, size_t keep) {
+  const std::lock_guard<std::mutex> guard(p.lock);
+  uint64_t used = 0;
+  if (keep) cudaMemPoolGetAttribute(p.pool, cudaMemPoolAttrUsedMemCurrent, &used);
+  return cudaMemPoolTrimTo(p.pool, keep ? used + keep : 0);
 }
 
 cudaError_t ensure_pool(cb_ctx* ctx) {
   if (ctx->pool || !ctx->pooled) return cudaSuccess;
-  cudaMemPoolProps props = {};
-  props.allocType = cudaMemAllocationTypePinned;
-  props.location.type = cudaMemLocationTypeDevice;
-  props.location.id = ctx->device;
-  cudaDeviceProp dp;
-  cudaError_t e = cudaGetDeviceProperties(&dp, ctx->device);
-  if (e == cudaSuccess && !(ctx->pool = reuse_pool(ctx->device))) e = cudaMemPoolCreate(&ctx->pool, &props);
-  if (e != cudaSuccess) {
-    ctx->pool = nullptr;
-    return e;
+  cb::DevicePool& p = device_pool(ctx->device);
+  const std::lock_guard<std::mutex> guard(p.lock);
+  uint64_t used = 0;
+  if (p.pool && !p.contexts &&
+      cudaMemPoolGetAttribute(p.pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess) {
+    (void)cudaGetLastError();  // the device was reset since
+    p.pool = nullptr;
   }
-  ctx->pool_idle_max = dp.totalGlobalMem / kIdleShare;
-  uint64_t hold = ctx->pool_idle_max;
-  return cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &hold);
+  if (!p.pool) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = ctx->device;
+    const OnDevice on(ctx->device);
+    size_t free_b = 0;
+    cudaError_t e = cudaMemGetInfo(&free_b, &p.total);
+    if (e == cudaSuccess) e = cudaMemPoolCreate(&p.pool, &props);
+    if (e != cudaSuccess) {
+      p.pool = nullptr;
+      return e;
+    }
+    // no stream waits for another one's memory (the default would let it)
+    int no = 0;
+    cudaMemPoolSetAttribute(p.pool, cudaMemPoolReuseAllowInternalDependencies, &no);
+  }
+  ctx->pool = &p;
+  ++p.contexts;
+  set_bound(p, ctx->device);
+  return cudaSuccess;
 }
 
-// Bounds the pool's idle memory, counted beside what is in use now: the
-// release threshold covers both, and memory above it is returned at the next
-// synchronisation.  Called when a call ends and when C is freed; it acts once
-// kIdleMoved bytes have moved.
+// A context goes: its part of the idle memory cannot be told from the others',
+// so all of it is given back.
+void leave_pool(cb_ctx* ctx) {
+  if (!ctx->pool) return;
+  {
+    const std::lock_guard<std::mutex> guard(ctx->pool->lock);
+    --ctx->pool->contexts;
+    set_bound(*ctx->pool, ctx->device);
+  }
+  if (give_back(*ctx->pool, 0) != cudaSuccess) (void)cudaGetLastError();
+  ctx->pool = nullptr;
+}
+
+// Frees pool memory in stream order: cudaFree would leave it in the pool's
+// count of memory in use for good, and the bound too high by it.
+void free_pooled(void* p, cudaStream_t stream) {
+  if (!p || cudaFreeAsync(p, stream) == cudaSuccess) return;
+  (void)cudaGetLastError();
+  cudaFree(p);
+}
+
+// Bounds the pool's idle memory.  Called when a call ends and when C is freed;
+// it acts once kIdleMoved bytes have moved.
 void bound_idle(cb_ctx* ctx, size_t freed = 0) {
-  if (!ctx->pool || (ctx->pool_moved += freed) < kIdleMoved) return;
-  ctx->pool_moved = 0;
-  uint64_t used = 0, reserved = 0;
-  if (cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess ||
-      cudaMemPoolGetAttribute(ctx->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess)
-    return;
-  uint64_t idle = ctx->pool_idle_max;
-  size_t free_b = 0, total_b = 0;
-  if (reserved > used + kIdleUnchecked && cudaMemGetInfo(&free_b, &total_b) == cudaSuccess)
-    idle = std::min<uint64_t>(idle, std::max<uint64_t>(free_b / 2, kIdleUnchecked));
-  uint64_t hold = used + idle;
-  cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &hold);
+  if (!ctx->pool || (ctx->pool->moved += freed) < kIdleMoved) return;
+  const std::lock_guard<std::mutex> guard(ctx->pool->lock);
+  set_bound(*ctx->pool, ctx->device);
 }
 
 struct IdleBound {
@@ -198,13 +248,13 @@ cudaError_t dev_alloc(cb_ctx* ctx, T** p, size_t bytes) {
   if (!ctx->pooled) return cudaMallocAsync(q, bytes, ctx->stream);
   cudaError_t e = ensure_pool(ctx);
   if (e != cudaSuccess) return e;
-  ctx->pool_moved += bytes;
-  e = cudaMallocFromPoolAsync(q, bytes, ctx->pool, ctx->stream);
-  if (e == cudaErrorMemoryAllocation) {  // in pieces of the wrong sizes, maybe: start over
+  ctx->pool->moved += bytes;
+  e = cudaMallocFromPoolAsync(q, bytes, ctx->pool->pool, ctx->stream);
+  if (e == cudaErrorMemoryAllocation) {  // idle in pieces of the wrong sizes, or freed but pending: start over
     (void)cudaGetLastError();
-    if ((e = cudaStreamSynchronize(ctx->stream)) != cudaSuccess) return e;
-    if ((e = cudaMemPoolTrimTo(ctx->pool, 0)) != cudaSuccess) return e;
-    e = cudaMallocFromPoolAsync(q, bytes, ctx->pool, ctx->stream);
+    if ((e = cudaDeviceSynchronize()) != cudaSuccess) return e;
+    give_back(*ctx->pool, 0);
+    e = cudaMallocFromPoolAsync(q, bytes, ctx->pool->pool, ctx->stream);
   }
   return e;
 }
@@ -1699,9 +1749,9 @@ int cb_ctx_create(cb_ctx** out, void* stream) {
 
 void cb_ctx_destroy(cb_ctx* ctx) {
   if (!ctx) return;
-  if (ctx->ws || ctx->ws2) cudaStreamSynchronize(ctx->stream);
-  if (ctx->ws) cudaFree(ctx->ws);
-  if (ctx->ws2) cudaFree(ctx->ws2);
+  free_pooled(ctx->ws, ctx->stream);
+  free_pooled(ctx->ws2, ctx->stream);
+  if (ctx->pool || ctx->ws || ctx->ws2) cudaStreamSynchronize(ctx->stream);
   if (ctx->host) cudaFreeHost(ctx->host);
   if (ctx->fstat || ctx->fsync) cudaStreamSynchronize(ctx->stream);
   if (ctx->fstat) cudaFree(ctx->fstat);
@@ -1711,7 +1761,7 @@ void cb_ctx_destroy(cb_ctx* ctx) {
   if (ctx->spa_bits) cudaFree(ctx->spa_bits);
   for (cudaEvent_t e : ctx->ev)
     if (e) cudaEventDestroy(e);
-  retire_pool(ctx);  // arrays of C still in use keep their part of it until they are freed
+  leave_pool(ctx);  // arrays of C still in use keep their part of the pool until they are freed
   delete ctx;
 }
 
@@ -1873,11 +1923,23 @@ int cb_spgemm(cb_semiring sr, const cb_csr* A, const cb_csr* B, cb_csr* C) {
 
 void cb_csr_free(cb_csr* C) {
   if (!C) return;
-  if (C->row_ptr || C->col || C->val) cudaDeviceSynchronize();
-  if (C->row_ptr) cudaFree(C->row_ptr);
-  if (C->col) cudaFree(C->col);
-  if (C->val) cudaFree(C->val);
+  void* const arrays[] = {C->row_ptr, C->col, C->val};
   std::memset(C, 0, sizeof *C);
+  int device = -1;
+  for (void* p : arrays) {
+    cudaPointerAttributes at{};
+    if (!p) continue;
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess && at.type == cudaMemoryTypeDevice) device = at.device;
+    else (void)cudaGetLastError();
+  }
+  if (device < 0) return;  // nothing to free
+  const OnDevice on(device);
+  cudaDeviceSynchronize();
+  for (void* p : arrays) free_pooled(p, nullptr);
+  cudaStreamSynchronize(nullptr);
+  cb::DevicePool& pool = device_pool(device);
+  const std::lock_guard<std::mutex> guard(pool.lock);
+  if (pool.pool) set_bound(pool, device, true);
 }
 
 int cb_csr_free_async(cb_ctx* ctx, cb_csr* C) {
