@@ -185,6 +185,17 @@ int cb_ctx_create(cb_ctx **ctx, void *cuda_stream);
 void cb_ctx_destroy(cb_ctx *ctx);
 /* Rebind the context to another stream. */
 int cb_ctx_set_stream(cb_ctx *ctx, void *cuda_stream);
+/* Idle memory.  The contexts of a device allocate C and their workspaces from
+ * one pool of the library, which keeps memory that was freed for the next
+ * call: at most a quarter of the device's memory, and at most half of what is
+ * free beside it (or 1 GiB, if that is more).  Other allocations of the same
+ * process get idle memory when nothing else is free; all of it goes back to
+ * the system when a context is destroyed.  cb_ctx_trim gives it back at any
+ * time (before other processes need the device, say): it waits for ctx's
+ * stream and returns what the pool of ctx's device holds idle beyond
+ * keep_bytes (>= 0, else CB_ERR_ARG).  Memory freed on other streams is idle
+ * once their work has finished.  cb_spgemm keeps nothing. */
+int cb_ctx_trim(cb_ctx *ctx, int64_t keep_bytes);
 const char *cb_last_error(const cb_ctx *ctx);
 const char *cb_status_str(int status);
 

@@ -98,6 +98,7 @@ _SIGS = {
     "cb_ctx_create": ([ctypes.POINTER(c_void_p), c_void_p], ctypes.c_int),
     "cb_ctx_destroy": ([c_void_p], None),
     "cb_ctx_set_stream": ([c_void_p, c_void_p], ctypes.c_int),
+    "cb_ctx_trim": ([c_void_p, c_int64], ctypes.c_int),
     "cb_last_error": ([c_void_p], ctypes.c_char_p),
     "cb_status_str": ([ctypes.c_int], ctypes.c_char_p),
     "cb_spgemm": ([ctypes.c_int, ctypes.POINTER(cb_csr), ctypes.POINTER(cb_csr),
@@ -320,6 +321,13 @@ class Context:
     def check(self, rc: int):
         if rc != 0:
             raise CBError(rc, self.error())
+
+    def trim(self, keep_bytes: int = 0) -> None:
+        """Give the idle memory of the device's pool, beyond keep_bytes, back to
+        the system (cb_ctx_trim)."""
+        rc = self.lib.cb_ctx_trim(self.handle, int(keep_bytes))
+        if rc != 0:
+            raise CBError(rc, "cb_ctx_trim failed")
 
     def set_tune(self, sym_hash_max=512, num_hash_max=512, learn_max=512, cf_esc=1.25,
                  cf_prereduce=4.0) -> dict:

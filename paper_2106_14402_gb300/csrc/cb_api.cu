@@ -1775,6 +1775,13 @@ int cb_ctx_set_stream(cb_ctx* ctx, void* stream) {
   return CB_OK;
 }
 
+int cb_ctx_trim(cb_ctx* ctx, int64_t keep_bytes) {
+  if (!ctx || keep_bytes < 0) return CB_ERR_ARG;
+  if (cudaStreamSynchronize(ctx->stream) != cudaSuccess) return CB_ERR_CUDA;
+  if (!ctx->pool) return CB_OK;
+  return give_back(*ctx->pool, (size_t)keep_bytes) == cudaSuccess ? CB_OK : CB_ERR_CUDA;
+}
+
 const char* cb_last_error(const cb_ctx* ctx) { return ctx ? ctx->err.c_str() : "null context"; }
 
 const char* cb_status_str(int s) {

@@ -1,6 +1,6 @@
 """Idle memory of the library's pool with most of the device taken: the bound
-holds by whichever function, context and order C is freed, and other
-allocations of the process get what is idle."""
+holds by whichever function, context and order C is freed, a caller can have
+it given back, and other allocations of the process get what is idle."""
 import ctypes
 import gc
 
@@ -112,3 +112,21 @@ def test_other_allocations_get_idle_memory(cb, big, others):
     cb.spgemm(SR, dA, dA, ctx=ctx)
     assert before - free_bytes() >= c_bytes
     others(-c_bytes // 2)                      # half of C more than is free
+
+
+def test_trim_gives_idle_memory_back(cb, big):
+    dA, c_bytes = big
+    ctx = cb.Context()
+    before = free_bytes()
+    C = cb.spgemm(SR, dA, dA, ctx=ctx)
+    in_use = before - free_bytes() - c_bytes
+    del C
+    for keep in (1 << 30, 0):
+        ctx.trim(keep)
+        assert before - free_bytes() <= in_use + keep + 64 * MB
+    C = cb.spgemm(SR, dA, dA, ctx=ctx)         # what is in use stays
+    ctx.trim()
+    assert 12 * C.nnz == c_bytes and int(C.row_ptr[-1]) == C.nnz
+    with pytest.raises(cb.CBError):
+        ctx.trim(-1)
+    cb.Context().trim()                        # nothing allocated yet
