@@ -233,6 +233,15 @@ void bound_idle(cb_ctx* ctx, size_t freed = 0) {
   set_bound(*ctx->pool, ctx->device);
 }
 
+// What the context's pool holds idle.
+size_t idle_bytes(cb_ctx* ctx) {
+  uint64_t used = 0, reserved = 0;
+  if (!ctx->pool || cudaMemPoolGetAttribute(ctx->pool->pool, cudaMemPoolAttrUsedMemCurrent, &used) != cudaSuccess ||
+      cudaMemPoolGetAttribute(ctx->pool->pool, cudaMemPoolAttrReservedMemCurrent, &reserved) != cudaSuccess)
+    return 0;
+  return reserved > used ? reserved - used : 0;
+}
+
 struct IdleBound {
   cb_ctx* ctx;
   ~IdleBound() { bound_idle(ctx); }
@@ -742,11 +751,12 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, DevCSR dB, int64_t out_n
   const int64_t win_cap = wcut.most(n_heavy * spans, cb::kSpanWords, ctx->stats.flops);
 
   // Heavy-row bitmaps are kept for the numeric phase when they fit a quarter
-  // of free device memory (capped at 32 GiB); otherwise the numeric phase
-  // rebuilds each window's bitmap from the products.
+  // of free device memory (capped at 32 GiB), the pool's idle memory included;
+  // otherwise the numeric phase rebuilds each window's bitmap from the products.
   const size_t bits_bytes = (size_t)(n_heavy * spans) * cb::kSpanWords * sizeof(unsigned);
   size_t free_b = 0, total_b = 0;
   CB_CUDA(cudaMemGetInfo(&free_b, &total_b));
+  free_b += idle_bytes(ctx);
   const bool keep_bits = n_heavy > 0 && bits_bytes <= free_b / 4 && bits_bytes <= (32ull << 30);
   const size_t racc_bytes = n_heavy > 0 ? cb::rank_scratch_bytes(sr, ctx->sms) : 0;
   // rank windows that cover part of a row slice B's rows by a split table

@@ -130,3 +130,24 @@ def test_trim_gives_idle_memory_back(cb, big):
     with pytest.raises(cb.CBError):
         ctx.trim(-1)
     cb.Context().trim()                        # nothing allocated yet
+
+
+def test_idle_memory_counts_as_free_for_the_bitmaps(cb, big, others):
+    """A second call keeps the heavy rows' bitmaps (and with them the (or,and)
+    read-out, one launch less) where the first one did, although the first
+    one's C is now idle memory."""
+    P, _ = big
+    A = cb.DeviceCSR(P.nrows, P.ncols, P.row_ptr, P.col, torch.ones(P.nnz, dtype=torch.uint8, device="cuda"))
+    bits = 32768 * int((cb.row_stats(A, A)[0].clamp(max=P.ncols) > 512).sum())
+    before = free_bytes()
+    ctx = cb.Context()
+    C = cb.spgemm("or_and_bool", A, A, ctx=ctx)
+    want, c_bytes = ctx.stats()["kernels"], 5 * C.nnz
+    in_use = before - free_bytes() - c_bytes
+    assert in_use >= bits
+    del C, ctx
+    ctx = cb.Context()
+    others(4 * bits + in_use + c_bytes // 4)
+    for _ in range(2):
+        cb.spgemm("or_and_bool", A, A, ctx=ctx)
+        assert ctx.stats()["kernels"] == want
