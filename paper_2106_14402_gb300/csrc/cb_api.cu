@@ -759,14 +759,10 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, DevCSR dB, int64_t out_n
   free_b += idle_bytes(ctx);
   const bool keep_bits = n_heavy > 0 && bits_bytes <= free_b / 4 && bits_bytes <= (32ull << 30);
   const size_t racc_bytes = n_heavy > 0 ? cb::rank_scratch_bytes(sr, ctx->sms) : 0;
-  // rank windows that cover part of a row slice B's rows by a split table
-  size_t tab_bytes = 0;
-  cb::SplitTable tab;
-  if (n_heavy > 0 && b_sorted) tab = cb::split_table_shape(dB.nrows, ncols, &tab_bytes);
   size_t need2 = align_up(4 * (size_t)(n_heavy * spans) + 4) +
                  align_up(8 * (size_t)(n_heavy * spans) + 8) +
                  align_up(sizeof(cb::Window) * (size_t)win_cap) + (keep_bits ? align_up(bits_bytes) : 0) +
-                 align_up(racc_bytes) + align_up(tab_bytes);
+                 align_up(racc_bytes);
   ensure(ctx, &ctx->ws2, &ctx->ws2_cap, need2);
   Carver cv2{static_cast<char*>(ctx->ws2)};
   int32_t* span_counts = cv2.take<int32_t>(n_heavy * spans + 1);
@@ -774,7 +770,6 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, DevCSR dB, int64_t out_n
   cb::Window* wins = cv2.take<cb::Window>(win_cap);
   unsigned* hbits = keep_bits ? cv2.take<unsigned>((size_t)(n_heavy * spans) * cb::kSpanWords) : nullptr;
   void* racc = racc_bytes ? cv2.take<char>(racc_bytes) : nullptr;
-  int32_t* tab_pos = tab_bytes ? cv2.take<int32_t>(tab_bytes / 4) : nullptr;
   const int32_t* heavy_rows = perm_sym + sym_beg[cb::kSymHeavy];
 
   int launches = 0;
@@ -840,12 +835,22 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, DevCSR dB, int64_t out_n
 
   launches = 0;
   mark(ctx, opt, 4);
-  // a pass over B's rows for the table pays once more than a few rows are cut
-  // into several windows (a row's only window takes B's rows whole)
-  if (tab_pos && !pattern && n_units > n_heavy + n_heavy / 8) {
-    tab.pos = tab_pos;
-    cb::launch_split_table(dB, tab, ctx->stream, ctx->sms);
-    ++launches;
+  // Rank windows that cover part of a row slice B's rows by a split table.  A
+  // pass over B's rows for it pays once more than a few rows are cut into
+  // several windows (a row's only window takes B's rows whole).  Without memory
+  // for it the windows search whole rows.
+  DevBuf tab_buf(ctx);
+  cb::SplitTable tab;
+  if (b_sorted && !pattern && n_units > n_heavy + n_heavy / 8) {
+    size_t bytes = 0;
+    tab = cb::split_table_shape(dB.nrows, ncols, &bytes);
+    if (bytes && dev_alloc(ctx, &tab_buf.p, bytes) == cudaSuccess) {
+      tab.pos = tab_buf.as<int32_t>();
+      cb::launch_split_table(dB, tab, ctx->stream, ctx->sms);
+      ++launches;
+    } else if (bytes) {
+      (void)cudaGetLastError();
+    }
   }
   if (pattern) {
     cb::launch_pattern_rows(dA, dB, heavy_rows, n_heavy, spans, span_counts, hbits, nnz, C->row_ptr, C->col,

@@ -132,7 +132,7 @@ void launch_slabs(const DevCSR& B, const int64_t* bnd, int nb1, int64_t* pos, cu
                   int sms);
 
 // Shape of a split table for a view of n rows and ncols columns (pos unset)
-// and its bytes; stride 0 where a table would not pay.
+// and its bytes; stride 0 and no bytes where a table would not pay.
 SplitTable split_table_shape(int64_t n, int64_t ncols, size_t* bytes);
 // Fills the table t (t.pos is device memory of that size); B's rows must be sorted.
 void launch_split_table(const DevCSR& B, const SplitTable& t, cudaStream_t s, int sms);

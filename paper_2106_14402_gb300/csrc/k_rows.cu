@@ -220,9 +220,12 @@ __global__ void __launch_bounds__(256) k_tier_scatter(int64_t m, TierBySize tier
 // sectors instead of eleven probes all over the row).  R-MAT s18 numeric: f64
 // 47.5 -> 46.2 ms, u32 36.8 -> 34.0, the table (68 MB) included.  Boundaries
 // lie 2^kSplitShift columns apart, further where the table would exceed
-// kSplitMaxBytes.
+// kSplitMaxBytes; there is none where that leaves fewer than kSplitLeast parts
+// of a row (each doubling of the distance costs every search one more probe,
+// and four parts save two).
 constexpr int kSplitShift = 12;
 constexpr int64_t kSplitMaxBytes = int64_t(256) << 20;
+constexpr int64_t kSplitLeast = 4;
 __global__ void __launch_bounds__(256) k_split_table(DevCSR B, int stride, int shift, int32_t* pos) {
   const int lane = threadIdx.x & 31;
   const int64_t nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
@@ -427,7 +430,10 @@ SplitTable split_table_shape(int64_t n, int64_t ncols, size_t* bytes) {
   t.shift = kSplitShift;
   if (ncols <= (int64_t(1) << t.shift)) return t;
   const auto size = [&] { return ((ncols + (int64_t(1) << t.shift) - 1) >> t.shift) + 1; };
-  while (size() * n * 4 > kSplitMaxBytes && t.shift < 30) ++t.shift;
+  while (size() * n * 4 > kSplitMaxBytes) {
+    ++t.shift;
+    if (size() <= kSplitLeast) return SplitTable{};
+  }
   t.stride = (int)size();
   *bytes = (size_t)t.stride * (size_t)n * 4;
   return t;
