@@ -636,7 +636,8 @@ bool try_fused_speculatively(cb_ctx* ctx, int sr, const DevCSR& dA, int64_t a_nn
 // skip (optional): rows already computed elsewhere; their sizes are preset[i]
 // and the exact phases leave them out.
 // a_rcols (optional): per-row output width of A's rows (stacked batches).
-// b_nnz (optional, >= 0): B's stored entries, for the speculative one-launch path.
+// b_nnz (optional, >= 0): B's stored entries, for the speculative one-launch path
+// and the split table's limit.
 // A validation queued by the caller (ctx->validating) is checked at the first
 // synchronisation.
 void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, DevCSR dB, int64_t out_ncols,
@@ -837,11 +838,14 @@ void spgemm_plain(cb_ctx* ctx, int sr, const cb_csr* A, DevCSR dB, int64_t out_n
   mark(ctx, opt, 4);
   // Rank windows that cover part of a row slice B's rows by a split table.  A
   // pass over B's rows for it pays once more than a few rows are cut into
-  // several windows (a row's only window takes B's rows whole).  Without memory
-  // for it the windows search whole rows.
+  // several windows (a row's only window takes B's rows whole).  Its positions
+  // in a row are 32-bit: a row that A names has at most as many entries as some
+  // row of C has products, and at most B's.  Without memory for it the windows
+  // search whole rows.
   DevBuf tab_buf(ctx);
   cb::SplitTable tab;
-  if (b_sorted && !pattern && n_units > n_heavy + n_heavy / 8) {
+  if (b_sorted && !pattern && n_units > n_heavy + n_heavy / 8 &&
+      (ctx->host[cb::kMaxFlops] <= INT32_MAX || (b_nnz >= 0 && b_nnz <= INT32_MAX))) {
     size_t bytes = 0;
     tab = cb::split_table_shape(dB.nrows, ncols, &bytes);
     if (bytes && dev_alloc(ctx, &tab_buf.p, bytes) == cudaSuccess) {

@@ -71,3 +71,21 @@ def test_table_shapes(cb, sr, n, ncols, spread):
     # workspaces without a table, the 8-byte windows' slices among them (three
     # CTAs an SM, 16384 entries of 8 bytes, a quarter to spare)
     assert before - free_bytes() <= 64 * MB + 3 * 152 * 16384 * 8 * 5 // 4
+
+
+def test_rows_beyond_32_bit_positions(cb):
+    """A row of more than 2^31 entries (2048 of each column): no table, whose
+    positions in a row are 32-bit."""
+    n, each = (1 << 20) + 1, 2048
+    nnz = n * each
+    assert nnz > 1 << 31
+    col = torch.arange(n, dtype=torch.int32, device="cuda")
+    val = (col % 1000 + 1).repeat_interleave(each)
+    val.view(n, each)[:, -1] -= 1              # the smallest of each column comes last
+    B = cb.DeviceCSR(1, n, torch.tensor([0, nnz], device="cuda"), col.repeat_interleave(each), val.view(torch.uint32))
+    A = cb.DeviceCSR(2, 1, torch.tensor([0, 1, 2], device="cuda"), torch.zeros(2, dtype=torch.int32, device="cuda"),
+                     torch.tensor([5, 7], dtype=torch.int32, device="cuda").view(torch.uint32))
+    C = cb.spgemm("min_plus_u32", A, B, ctx=cb.Context())
+    assert C.row_ptr.tolist() == [0, n, 2 * n]
+    assert torch.equal(C.col, torch.cat([col, col]))
+    assert torch.equal(C.val.view(torch.int32), torch.cat([col % 1000 + 5, col % 1000 + 7]))
