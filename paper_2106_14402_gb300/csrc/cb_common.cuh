@@ -261,7 +261,7 @@ template <> struct Sem<7> {
 //     windows exist.
 // A rank window is a run of whole bitmap words of one span that fits the
 // numeric kernel's shared memory (num_window_cut); inside it an output column's slot is
-// its rank (popcount of the set bits before it), so a dense array of kWcap
+// its rank (popcount of the set bits before it), so a dense array of
 // accumulators indexed by rank holds the window and reads out sorted.
 // ---------------------------------------------------------------------------
 constexpr int kEmptyKey = -1;
@@ -800,8 +800,8 @@ __device__ __forceinline__ void for_row_pieces(const DevCSR& A, const DevCSR& B,
       sm.len[slot] = (int)(q1 - q0);
     }
     __syncthreads();
-    // equal runs of pieces per warp; nwarp is a power of two (512- and
-    // 1024-thread CTAs), so the split needs no 64-bit division
+    // equal runs of pieces per warp; nwarp is a power of two (512-thread
+    // CTAs), so the split needs no 64-bit division
     const int lgw = 31 - __clz(nwarp);
     const int k_beg = (int)((npieces * warp) >> lgw), k_end = (int)((npieces * (warp + 1)) >> lgw);
     if (k_beg < k_end) {  // uniform over the warp
