@@ -1864,6 +1864,7 @@ int cb_spgemm_ex(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_csr* B, 
     return CB_OK;
   } catch (const Fail& f) {
     ctx->validating = false;
+    if (caller_buf && C && f.code == CB_ERR_INDEX) *C = saved;  // an invalid operand leaves C alone
     if (!caller_buf && C) {
       if (C->row_ptr && C->row_ptr != saved.row_ptr) cudaFreeAsync(C->row_ptr, ctx->stream);
       if (C->col && C->col != saved.col) cudaFreeAsync(C->col, ctx->stream);

@@ -65,3 +65,21 @@ def test_bad_index_is_caught_before_use(cb, deg, bad, off):
     assert bool((out.col == -7).all()) and bool((out.row_ptr == -7).all())
     (target.row_ptr if "row_ptr" in bad else target.col).copy_(saved)
     compare_rows(SR, cb.spgemm(SR, dA, dB, ctx=ctx).to_host(), want)
+
+
+@pytest.mark.parametrize("deg", [4, 40, 120])
+def test_caller_struct_is_untouched(cb, deg):
+    """A failed validation leaves every field of a caller-provided C as it was."""
+    import ctypes
+    n = 2001
+    A = gen.er_exact(n, n, deg, 924)
+    dA = operand(cb, A.with_values(gen.random_values(SR, A.nnz, 925)))
+    dA.col[A.nnz - 1] = n
+    rp, col = (torch.empty(k, dtype=t, device="cuda") for k, t in ((n + 1, torch.int64), (9, torch.int32)))
+    sa, opts = dA.as_struct(), cb.make_opts(out_capacity=9)
+    sc = cb.cb_csr(11, 12, 13, rp.data_ptr(), col.data_ptr(), col.data_ptr())
+    ctx = cb.Context()
+    rc = ctx.lib.cb_spgemm_ex(ctx.handle, 3, ctypes.byref(sa), ctypes.byref(sa), ctypes.byref(sc), ctypes.byref(opts))
+    assert rc == CB_ERR_INDEX
+    assert (sc.nrows, sc.ncols, sc.nnz) == (11, 12, 13)
+    assert (sc.row_ptr, sc.col, sc.val) == (rp.data_ptr(), col.data_ptr(), col.data_ptr())
