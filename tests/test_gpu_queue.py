@@ -125,3 +125,18 @@ def test_queue_row_that_never_publishes(cb, row):
     ctx.set_fault(cb.FAULT_SILENT_TILE, -1)
     C = cb.spgemm(sr, dA, dB, ctx=ctx)
     compare_rows(sr, C.to_host(), oracle.spgemm(sr, A, B))
+
+
+@pytest.mark.parametrize("deg", [40, 60])
+def test_queue_rows_signs_of_zero(cb, deg):
+    """Sums start at +0.0, a single product of -0.0 included (small whole
+    values, so every sum is exact and compared bit for bit)."""
+    sr = "plus_times_f64"
+    A, B = er_pair(sr, 3000, deg, deg, seed=640)
+    rng = np.random.default_rng(641)
+    A, B = (M.with_values(rng.choice([-2.0, -1.0, -0.0, 0.0, 1.0], M.nnz)) for M in (A, B))
+    got, st = run(cb, sr, A, B)
+    assert st["kernels"] == 6
+    want = oracle.spgemm(sr, A, B)
+    assert not np.signbit(want[2][want[2] == 0]).any()
+    assert np.array_equal(got[2].view(np.int64), np.asarray(want[2], np.float64).view(np.int64))
