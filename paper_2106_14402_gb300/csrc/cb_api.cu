@@ -2149,6 +2149,7 @@ int cb_spmspv(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_spvec* x, c
   cb_spvec saved{};
   if (y) saved = *y;
   const IdleBound bound{ctx};
+  bool filled = false;  // the accumulator holds products that the compaction has not taken out
   try {
     if (!A || !x || !y) fail(ctx, CB_ERR_ARG, "null argument");
     if (!public_semiring(sr)) fail(ctx, CB_ERR_SEMIRING, "unknown semiring");
@@ -2226,6 +2227,7 @@ int cb_spmspv(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_spvec* x, c
                            nullptr, nullptr, nullptr, nullptr, 0, counters + cb::kError, ctx->stream,
                            ctx->sms);
     cb::launch_exclusive_scan(chunks, nx, cpre, partial, ctx->stream);
+    filled = true;
     cb::launch_spmspv_step((int)sr, 2, dA, x->idx, x->val, nx, nullptr, cpre, ctx->spa, ctx->spa_bits, n,
                            nullptr, nullptr, nullptr, nullptr, 0, nullptr, ctx->stream, ctx->sms);
     cb::launch_spmspv_step((int)sr, 3, dA, nullptr, nullptr, 0, nullptr, nullptr, nullptr, ctx->spa_bits,
@@ -2248,6 +2250,7 @@ int cb_spmspv(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_spvec* x, c
                            ctx->spa_bits, n, nullptr, wpre, y->idx, y->val, std::min(cap, total),
                            nullptr, ctx->stream, ctx->sms);
     CB_LAUNCHED();
+    filled = false;
     ctx->stats.kernels += 1;
     mark(ctx, opt, 2);
     mark(ctx, opt, 3);
@@ -2266,6 +2269,7 @@ int cb_spmspv(cb_ctx* ctx, cb_semiring sr, const cb_csr* A, const cb_spvec* x, c
     collect_times(ctx, opt, true);
     return CB_OK;
   } catch (const Fail& f) {
+    if (filled) ctx->spa_n = 0;  // the next call starts with a new one
     if (!caller_buf && y) {
       if (y->idx && y->idx != saved.idx) cudaFreeAsync(y->idx, ctx->stream);
       if (y->val && y->val != saved.val) cudaFreeAsync(y->val, ctx->stream);

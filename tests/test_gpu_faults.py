@@ -212,3 +212,33 @@ def test_allocation_failures_batched(cb):
 
     failures, _ = _oom_sweep(cb, run, check, kmax=40)
     assert failures >= 3, failures
+
+
+def test_allocation_failures_spmspv(cb):
+    """A call that fails after its products were combined leaves none of them
+    to the next one."""
+    sr = "min_plus_u32"
+    A = gen.random_csr(300, 5000, 0.02, seed=650, semiring=sr)
+    dA = cb.DeviceCSR.from_host(A, sr)
+
+    def run(ctx, first):
+        idx = np.arange(first, 300, 7).astype(np.int32)
+        val = np.full(idx.size, 10 - first, np.uint32)
+        yi, yv = cb.spmspv(sr, dA, torch.from_numpy(idx).cuda(),
+                           torch.from_numpy(val.view(np.int32)).cuda().view(torch.uint32), ctx=ctx)
+        wi, wv, _ = oracle.spmspv(sr, A, idx, val)
+        assert np.array_equal(yi.cpu().numpy(), wi)
+        assert np.array_equal(yv.view(torch.int32).cpu().numpy().view(np.uint32), wv)
+
+    for k in range(1, 13):
+        ctx = cb.Context()
+        ctx.set_fault(cb.FAULT_ALLOC, k)
+        try:
+            run(ctx, 3)
+        except cb.CBError as e:
+            assert e.code == CB_ERR_OOM
+            run(ctx, 0)
+            continue
+        assert k > 4                           # workspace, accumulator, y's indices and values
+        return
+    raise AssertionError("every allocation up to 12 failed")
