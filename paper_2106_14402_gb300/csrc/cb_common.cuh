@@ -269,7 +269,7 @@ constexpr int kEmptyKey = -1;
 constexpr int kSymWarpMax = 128;     // warp team, table <= 256 slots
 constexpr int kSymSmallMax = 512;    // 256-thread team, table <= 1024
 constexpr int kSymHashMax = 512;     // default bound of the hash tiers (runtime-tunable)
-constexpr int kSymLargeMax = 4096;   // largest bound the 1024-thread hash tier supports
+constexpr int kSymLargeMax = 4096;   // largest bound the 512-thread hash tier supports
 constexpr int kSpanCols = 1 << 18;   // columns per bitmap span
 constexpr int kSpanWords = kSpanCols / 32;
 constexpr int kMaxWindowsPerSpan = 64;

@@ -341,7 +341,8 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
   }
   // 8-byte accumulators reduce in L2 (a per-CTA slice of racc): shared-memory
   // 64-bit atomics cost more than L2 reductions, and without shared
-  // accumulators three 512-thread CTAs share an SM (40 registers each).
+  // accumulators three 512-thread CTAs share an SM (40 registers each, 20-24
+  // bytes of them spilled for int64, fp64, (or,and) and the merge form).
   constexpr bool kL2 = NumLimits<SR>::kL2Acc;
   // (+,x) over int64 and fp64 accumulate in L2 directly in the window's
   // output entries (their accumulator bits are the output value's), so the
@@ -372,7 +373,6 @@ __global__ void __launch_bounds__(CTA, RankShape<SR>::kPerSm) k_num_rank(DevCSR 
   __shared__ long long s_base;
   __shared__ long long next;
   const int tid = threadIdx.x, lane = tid & 31;
-  const TA* Aval = reinterpret_cast<const TA*>(A.val);
   const TB* Bval = reinterpret_cast<const TB*>(B.val);
 
   take_unit(queue, &next);

@@ -64,7 +64,9 @@ __device__ __forceinline__ typename Sem<SR>::A started(typename Sem<SR>::A y) {
   else return y;
 }
 
-constexpr int kQCtas = 8;  // per SM (64 registers a thread; 7 and 9 took 2% and 9% longer)
+// CTAs per SM: 64 registers a thread, 12 bytes of them spilled for int64 and
+// fp64 (7 and 9 took 2% and 9% longer).
+constexpr int kQCtas = 8;
 
 // status words: [63:40] epoch, [39:38] kind, [37:0] value (as in k_fused.cu)
 constexpr int kQEpochShift = 40;

@@ -205,7 +205,6 @@ __global__ void __launch_bounds__(256) k_tier_scatter(int64_t m, TierBySize tier
     base[threadIdx.x] =
         seg + (long long)atomicAdd((unsigned long long*)&cur[threadIdx.x], (unsigned long long)local[threadIdx.x]);
   }
-  __syncthreads();
   if (threadIdx.x == 5 && local[5])
     base[5] = cnt[1] + cnt[2] + cnt[3] + cnt[4] - 1 -
               (long long)atomicAdd((unsigned long long*)&tier.counters[kCurHeavy], (unsigned long long)local[5]);
