@@ -1962,8 +1962,9 @@ void cb_csr_free(cb_csr* C) {
   if (device < 0) return;  // nothing to free
   const OnDevice on(device);
   cudaDeviceSynchronize();
-  for (void* p : arrays) free_pooled(p, nullptr);
-  cudaStreamSynchronize(nullptr);
+  // (on the legacy stream the frees would break a capture on a blocking stream)
+  for (void* p : arrays) free_pooled(p, cudaStreamPerThread);
+  cudaStreamSynchronize(cudaStreamPerThread);
   cb::DevicePool& pool = device_pool(device);
   const std::lock_guard<std::mutex> guard(pool.lock);
   if (pool.pool) set_bound(pool, device, true);
